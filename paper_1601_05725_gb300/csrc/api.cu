@@ -32,6 +32,12 @@ struct basker_s {
     std::vector<size_t> lv_smem;
     std::vector<int32_t *> lv_cols;
     std::vector<int32_t> lv_ncols;
+    // the level-0 tasks (ND leaves, BTF blocks) factored by teams of warps
+    std::vector<bk_team_group> team;
+    bool team_path = false;      // every level-0 task has a team, every separator a dense elimination
+    bool stored_first = false;   // the stored-pattern pass before the teams (dense enough columns)
+    bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones)
+    bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once from then on
     // separators whose in-node phase runs as one dense elimination, by cluster size
     // ([0]: one block, [1]: BK_DENSE_CLUSTER blocks)
     std::vector<int32_t *> lv_dense[2];
@@ -44,6 +50,8 @@ struct basker_s {
     int32_t *h_task_fail = nullptr;  // pinned
     int32_t epoch = 0, solve_epoch = 0, refno = 0;
     bool factored = false, ws_dirty = false, schedule_valid = true, order_is_symbolic = true;
+    bool leaf_levels = false;    // the teams wrote the leaves' column levels (all the solve reads)
+    bool order_stale = false;    // the stored claim order does not belong to the stored levels
     double gp_wall_ms = 0.0;     // wall time of the last complete Algorithm 1 pass (host clock)
     double round_us_per_col = 0.0;   // a refactorization round's wall time per column it processed
     bool sep_dense = false;      // refactorizations recompute every separator densely
@@ -247,6 +255,7 @@ int alloc_factors(basker_t h)
     TRY(dalloc(h, &r.Urx, (size_t)h->d.upool_end));
     TRY(dalloc(h, &r.tk, (size_t)std::max(h->d.lpool_end, h->d.upool_end)));
     TRY(dalloc(h, &r.Ls, (size_t)h->d.lpool_end));
+    h->d.Ls = r.Ls;
     TRY(dalloc(h, &r.tx, (size_t)std::max(h->d.lpool_end, h->d.upool_end)));
     TRY(dalloc(h, &h->d.Lx, (size_t)h->d.lpool_end + 4));
     TRY(dalloc(h, &h->d.Ui, (size_t)h->d.upool_end));
@@ -333,6 +342,68 @@ int restore_symbolic_image(basker_t h, cudaStream_t s)
     int64_t *const b[4] = {d.Lbeg, d.Ubeg, d.Lend, d.Uend};
     for (int i = 0; i < 4; i++) CU(cudaMemcpyAsync(b[i], h->sym_beg + i * n, n * 8, cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(d.pool, h->sym_pool, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+    return BASKER_OK;
+}
+
+// The teams of the level-0 tasks.  A task of more than 1,024 rows (an ND leaf: few
+// tasks, the decisions' chain is the time) gets 16 warps; the others 16, 8 or 4 as
+// up to two or eight of them per SM, or more, share the GPU (factorization of
+// 4,096 netlist blocks 12.4 ms with 16 warps, 8.9 with 8, 7.3 with 4; 301 blocks
+// 3.0, 3.8 and 5.7 ms); a task of up to 16 rows one warp.  x in shared memory where
+// all the team's warps fit, else in the workspace slices.
+int setup_teams(basker_t h)
+{
+    const bk_plan &pl = h->pl;
+    h->team.clear();
+    std::vector<std::vector<int32_t>> ids;
+    if (pl.level_tasks.empty()) return BASKER_OK;
+    const int64_t slices = pl.level_warps.empty() ? 0 : pl.level_warps[0];
+    int32_t some = 0;
+    for (int32_t t : pl.level_tasks[0]) some += pl.tasks[(size_t)t].hi - pl.tasks[(size_t)t].lo > 16;
+    const int32_t wide = some <= 2 * 152 ? 16 : some <= 8 * 152 ? 8 : 4;
+    for (int32_t t : pl.level_tasks[0]) {
+        const bk_task &T = pl.tasks[(size_t)t];
+        const int32_t own = T.hi - T.lo;
+        if (own <= 0) continue;
+        bk_team_group g;
+        g.W = own <= 16 ? 1 : own <= 1024 ? wide : 16;
+        g.xs = bk_team_smem(T, g.W, true) <= BK_TEAM_SMEM;
+        while (g.W > 1 && (bk_team_smem(T, g.W, g.xs) > BK_TEAM_SMEM || (!g.xs && g.W > slices))) g.W /= 2;
+        if (own > 65534 || T.lspace > 65535 || T.sp_lo < T.lo || bk_team_smem(T, g.W, g.xs) > BK_TEAM_SMEM ||
+            (own > 16 && g.W < 4)) {
+            // tables too large: the handle keeps the paths without teams
+            h->team.clear();
+            return BASKER_OK;
+        }
+        size_t k = 0;
+        while (k < h->team.size() && !(h->team[k].W == g.W && h->team[k].xs == g.xs)) k++;
+        if (k == h->team.size()) {
+            h->team.push_back(g);
+            ids.emplace_back();
+        }
+        ids[k].push_back(t);
+        h->team[k].smem = std::max(h->team[k].smem, bk_team_smem(T, g.W, g.xs));
+    }
+    for (size_t k = 0; k < h->team.size(); k++) {
+        bk_team_group &g = h->team[k];
+        std::stable_sort(ids[k].begin(), ids[k].end(), [&](int32_t a, int32_t b) {
+            const bk_task &A = pl.tasks[(size_t)a], &B = pl.tasks[(size_t)b];
+            return A.hi - A.lo > B.hi - B.lo;
+        });
+        g.ntasks = (int32_t)ids[k].size();
+        g.smem = (g.smem + 15) & ~(size_t)15;
+        g.blocks = g.xs ? g.ntasks : (int32_t)std::max<int64_t>(1, std::min<int64_t>(g.ntasks, slices / g.W));
+        TRY(upload(h, &g.ids, ids[k]));
+    }
+    // the longest chains first
+    std::stable_sort(h->team.begin(), h->team.end(),
+                     [](const bk_team_group &a, const bk_team_group &b) { return a.W > b.W; });
+    bool sep = false;
+    for (const bk_task &T : pl.tasks) sep = sep || T.sp_lo < T.lo;
+    // Columns of 32 entries or more on average (power grids): the stored-pattern
+    // pass first, on every SM, and the teams only where it rejects pivots.
+    h->stored_first = !pl.counts_only && pl.nnz_l_sym + pl.nnz_u_sym >= (int64_t)32 * pl.n;
+    h->team_path = !h->team.empty() && (h->sep_dense || !sep) && h->opt.factor_mode == 0;
     return BASKER_OK;
 }
 
@@ -486,6 +557,7 @@ int setup_device(basker_t h)
         TRY(upload(h, &h->lv_cols[l], cols));
         h->lv_ncols[l] = (int32_t)cols.size();
     }
+    TRY(setup_teams(h));
     TRY(dalloc(h, &h->rd_tasks, (size_t)std::max<size_t>(pl.tasks.size(), 1)));
     TRY(dalloc(h, &h->rd_c0, (size_t)std::max<size_t>(pl.tasks.size(), 1)));
     TRY(dalloc(h, &h->rd_cols, (size_t)std::max(n, 1)));
@@ -640,10 +712,58 @@ int launch_desc_refactor(basker_t h, const int32_t *cols, int32_t ncols, cudaStr
     return BASKER_OK;
 }
 
+// Algorithm 1 on the level-0 tasks by teams (repair: from each task's first
+// rejected column on, after a stored-pattern pass).
+int launch_leaves(basker_t h, cudaStream_t s, int pref_mode, bool repair)
+{
+    if (!repair) CU(cudaMemsetAsync(h->d.pinv, 0xff, sizeof(int32_t) * (size_t)h->pl.n, s));
+    tbeg(h, repair ? KT_SPEC : KT_GP, s, (int)h->team.size());
+    for (const bk_team_group &g : h->team) {
+        bk_launch_team(level_dev(h, 0), g, h->opt.tau, pref_mode, h->opt.wait_budget_cycles, repair, s);
+        CU(cudaGetLastError());
+        h->launches++;
+    }
+    tend(h, s);
+    return BASKER_OK;
+}
+
+// The separators above level 0, level by level (Algorithm 4's dependency tree).
+// stored: the descendant phase starts from the stored patterns (verified on the
+// device), else every column takes the reach.
+int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
+{
+    for (size_t l = 1; l < h->lv_tasks.size(); l++) {
+        if (h->lv_ncols[l] > 0) {
+            if (stored) {
+                TRY(launch_desc_refactor(h, h->lv_cols[l], h->lv_ncols[l], s, l));
+            } else {
+                CU(cudaMemsetAsync(h->d.counter + 3, 0, sizeof(int32_t), s));
+                tbeg(h, KT_DESC, s, 1);
+                bk_launch_gp_desc(level_dev(h, l), h->lv_cols[l], h->lv_ncols[l], h->d.counter + 3, s);
+                CU(cudaGetLastError());
+                tend(h, s);
+                h->launches++;
+            }
+        }
+        for (int g = 0; g < 2; g++) {
+            if (h->lv_ndense[g][l] == 0) continue;
+            tbeg(h, KT_DENSE, s, 1);
+            bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], h->opt.tau, pref_mode,
+                                  g ? BK_DENSE_CLUSTER : 1, s);
+            CU(cudaGetLastError());
+            tend(h, s);
+            h->launches++;
+        }
+    }
+    return BASKER_OK;
+}
+
 // Algorithm 1 on every task, level by level (Algorithm 4's dependency tree).
 int launch_full_gp(basker_t h, cudaStream_t s, int pref_mode)
 {
     const double tau = h->opt.tau;
+    h->leaf_levels = false;
+    h->patterns_hold = true;       // nothing but a finished pass leads back to the teams
     CU(cudaMemsetAsync(h->d.pinv, 0xff, sizeof(int32_t) * (size_t)h->pl.n, s));
     for (size_t l = 0; l < h->lv_tasks.size(); l++) {
         if (l > 0 && h->lv_ncols[l] > 0) {
@@ -891,16 +1011,30 @@ int launch_repair_path(basker_t h, cudaStream_t s)
 
 int compute_schedule(basker_t h, cudaStream_t s)
 {
+    if (h->leaf_levels && h->team_path) {
+        // the teams left the leaves' levels, and the separators' columns wait for
+        // nothing in the stored-pattern pass: only the order by level is missing
+        tbeg(h, KT_LEVELS, s, 3);
+        bk_launch_order(h->d, s);
+        CU(cudaGetLastError());
+        tend(h, s);
+        h->launches += 3;
+        h->schedule_valid = true;
+        h->order_stale = false;
+        h->order_is_symbolic = false;
+        return BASKER_OK;
+    }
     h->epoch++;
     tbeg(h, KT_LEVELS, s, 5);
     // the stored levels are kept when they still order the new pattern (checked on
     // the device: a refactorization usually changes few columns)
-    bk_launch_levels(h->d, h->epoch, h->opt.wait_budget_cycles, static_blocks(h), s, true);
+    bk_launch_levels(h->d, h->epoch, h->opt.wait_budget_cycles, static_blocks(h), s, !h->order_stale);
     CU(cudaGetLastError());
     tend(h, s);
     h->launches += 5;
     CU(cudaGetLastError());
     h->schedule_valid = true;
+    h->order_stale = false;
     h->order_is_symbolic = false;
     return BASKER_OK;
 }
@@ -948,7 +1082,7 @@ int capture_finish(basker_t h)
 
 int finish_factorization(basker_t h, cudaStream_t s)
 {
-    if (!h->schedule_valid) TRY(compute_schedule(h, s));
+    if (!h->schedule_valid && !h->leaf_levels) TRY(compute_schedule(h, s));
     tbeg(h, KT_ROWS, s, 19);
     if (h->opt.graphs) {
         if (!h->g_finish || h->g_finish_ver != h->arena_ver) TRY(capture_finish(h));
@@ -1047,6 +1181,38 @@ int refactor_by_rounds(basker_t h, cudaStream_t s)
     return st;
 }
 
+// A factorization (pref_mode 0) or refactorization (1: the previous pivots, in
+// d.pref, preferred) with teams.  first: the stored-pattern pass runs first and
+// the teams repair its rejected pivots; else the teams compute every column.  The
+// separators follow, their descendant phase from the stored patterns (stored)
+// unless the leaves moved too many pivots for those to hold.  Returns the final
+// status; -1 for want of room.
+int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool &stored)
+{
+    const int32_t many = std::max(16, h->pl.n / 200);
+    if (first) {
+        if (!h->schedule_valid) TRY(compute_schedule(h, s));
+        TRY(static_pass(h, s));
+    }
+    h->schedule_valid = false;
+    TRY(launch_leaves(h, s, pref_mode, first));
+    if (h->lv_tasks.size() > 1 && stored && !pref_mode && !first) {
+        const int st = read_status(h, s);
+        if (st != BASKER_OK) return st;
+        stored = h->h_status->repaired <= many;
+    }
+    TRY(launch_separators(h, s, pref_mode, stored));
+    const int st = read_status(h, s);
+    h->patterns_hold = h->leaf_levels = st == BASKER_OK;
+    if (st == BASKER_OK && first && h->h_status->static_fail == 0) h->schedule_valid = true;   // no pattern moved
+    else h->order_stale = true;
+    if (st == BASKER_OK) {
+        note_repair(h);
+        if (first && h->h_status->static_fail > many) h->many_rejects = true;
+    }
+    return st;
+}
+
 int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
 {
     h->launches = 0;
@@ -1060,12 +1226,37 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         h->refno++;
         CU(cudaMemcpyAsync((void *)h->d.pref, h->d.prow, sizeof(int32_t) * (size_t)h->pl.n,
                            cudaMemcpyDeviceToDevice, s));
-        if (!h->schedule_valid) TRY(compute_schedule(h, s));
-        TRY(static_pass(h, s));
+        // options.refactor_switch 0, or 2 (the complete pass at once)
+        const bool teams = h->team_path && h->d.lpool_end < INT32_MAX && h->opt.refactor_switch % 2 == 0;
+        if (!teams) {
+            if (!h->schedule_valid) TRY(compute_schedule(h, s));
+            TRY(static_pass(h, s));
+            h->leaf_levels = false;
+        }
         h->info.last_repivot_columns = 0;
         h->info.last_rounds = 0;
         int st = BASKER_OK;
-        if (use_repair(h)) {
+        if (teams) {
+            bool stored = true;
+            const bool first = h->stored_first && h->patterns_hold && !h->many_rejects && h->opt.refactor_switch == 0;
+            st = factor_by_teams(h, s, 1, first, stored);
+            if (st == BASKER_ERR_TIMEOUT) {
+                // the pivots of before, for the next call
+                CU(cudaMemcpyAsync(h->d.prow, h->d.pref, sizeof(int32_t) * (size_t)h->pl.n,
+                                   cudaMemcpyDeviceToDevice, s));
+                return st;
+            }
+            for (int tries = 0; st == -1 && tries < 16; tries++) {
+                TRY(regrow(h));
+                TRY(reset_status(h, s));
+                stored = false;
+                st = factor_by_teams(h, s, 1, false, stored);
+            }
+            if (st == BASKER_OK && h->opt.refactor_switch == 2 && h->h_status->repaired > 0) {
+                h->info.full_refactors++;
+                h->info.last_rounds = 0;
+            }
+        } else if (use_repair(h)) {
             // the stored-pattern pass, the repair pass and the separators run back to
             // back on the device; the status is read once at the end
             TRY(launch_repair_path(h, s));
@@ -1088,7 +1279,49 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         h->factored = true;
         return BASKER_OK;
     }
-    int st = factor_static(h, s);
+    int st = BK_SWITCH_TO_FULL;
+    if (h->team_path && h->d.lpool_end < INT32_MAX) {
+        // from the symbolic arena (natural pivots and patterns) when it is there:
+        // the stored-pattern pass first, or at least the separators' patterns
+        bool stored = h->sym_Li && h->sym_ver == h->arena_ver && !h->static_factor_off && h->lv_tasks.size() > 1;
+        const bool first = stored && h->stored_first;
+        if (stored) {
+            TRY(restore_symbolic_image(h, s));
+            h->schedule_valid = true;
+            h->order_stale = false;
+            h->order_is_symbolic = true;
+            if (first) h->refno++;
+        }
+        const bool had = stored;
+        st = factor_by_teams(h, s, 0, first, stored);
+        if (st == BASKER_OK && had) {
+            if (first && h->h_status->static_fail > std::max(16, h->pl.n / 200)) {
+                h->static_factor_off = true;
+                h->many_rejects = false;         // the refactorizations' own count
+            } else if (!stored) {
+                h->static_factor_off = true;
+            }
+        }
+        for (int tries = 0; st == -1 && tries < 16; tries++) {
+            TRY(regrow(h));
+            TRY(reset_status(h, s));
+            stored = false;
+            st = factor_by_teams(h, s, 0, false, stored);
+        }
+        if (st == BASKER_OK) {
+            if (stored) h->info.static_factors++;
+            TRY(finish_factorization(h, s));
+            h->factored = true;
+            return BASKER_OK;
+        }
+        // a wait that gave up: the pass without waits below; a failure is final
+        if (st != BASKER_ERR_TIMEOUT) {
+            h->factored = false;
+            return st == -1 ? BASKER_ERR_OOM : st;
+        }
+    } else {
+        st = factor_static(h, s);
+    }
     if (st == BASKER_OK) {
         h->info.static_factors++;
         TRY(finish_factorization(h, s));

@@ -83,6 +83,8 @@ struct bk_dev {
     int64_t lpool_end, upool_end;    // array sizes: regions of the layout, then the pools
     int32_t *Li, *Ui;
     double *Lx, *Ux;
+    int32_t *Ls;                     // team kernel: the slots of L's rows in their task's L-space (the
+                                     // solve's row indices by column take the array afterwards)
     bk_status *status;
     int32_t *col_over;               // per column: 1 = its L region overflowed, 2 = its U region
     int32_t *task_stop;              // per task: nonzero once it or a descendant ran out of room
@@ -209,7 +211,25 @@ void bk_launch_static(const bk_dev &d, int32_t ncols, double tau, int32_t epoch,
                       long long budget, int blocks, void *stream);
 void bk_launch_levels(const bk_dev &d, int32_t epoch, long long budget, int blocks, void *stream,
                       bool check = false);
+// The claim order from the stored levels alone (levels valid, order not).
+void bk_launch_order(const bk_dev &d, void *stream);
 int bk_static_blocks();
+// kernels_team.cu: Algorithm 1 on tasks without descendants, a block of W warps per
+// task, columns in flight together, deciding in order
+#define BK_TEAM_SMEM (220 * 1024)
+struct bk_team_group {
+    int32_t *ids = nullptr;     // task ids (device), largest first
+    int32_t ntasks = 0;
+    int32_t W = 1;              // warps of a team (a power of two, at most 16)
+    int32_t blocks = 0;         // teams launched; each takes every blocks-th task
+    bool xs = false;            // x in shared memory (else in the warp's workspace slice)
+    size_t smem = 0;
+};
+size_t bk_team_smem(const bk_task &T, int W, bool xs);
+// repair: after the stored-pattern pass, from each task's first rejected column
+// (d.task_fail) on, columns that the changes do not reach kept as they stand
+void bk_launch_team(const bk_dev &d, const bk_team_group &g, double tau, int pref_mode, long long budget,
+                    bool repair, void *stream);
 // kernels_repair.cu: the rejected pivots of the ND leaves and BTF blocks resolved
 // in column order after the stored-pattern pass (one warp per task)
 size_t bk_repair_smem(const bk_task *tasks, const int32_t *ids, int32_t count, size_t limit);

@@ -88,6 +88,8 @@ __device__ __forceinline__ bool pattern_column(const bk_dev &d, const bk_task &T
     V *const Ux = vals<V>(d.Ux);
     const int base = T.sp_lo;
     const int own_lo = T.lo - base, own_hi = T.hi - base;
+    // the slots of L's rows, for the team kernel's repair (tasks without descendants)
+    const bool slots = base == T.lo;
     bool broken = false, bad = false;
     const int e1 = d.Bp[c + 1];
     for (int e = d.dstart[c] + lane; e < e1; e += 32) {
@@ -245,6 +247,7 @@ __device__ __forceinline__ bool pattern_column(const bk_dev &d, const bk_task &T
         if (fs[u] >= own_lo && fs[u] < own_hi) km = key_max(km, mag_key(v[u]));
         x[fs[u]] = 0.0;
         Lx[lb + lane + 32 * u] = v[u] / xp;
+        if (slots) d.Ls[lb + lane + 32 * u] = fs[u];
     }
     for (int t = 32 * FIX_PF + lane; t < lc; t += 32) {
         const int s = slot_of(T, base, d.Li[lb + t]);
@@ -254,6 +257,7 @@ __device__ __forceinline__ bool pattern_column(const bk_dev &d, const bk_task &T
         if (!isfinite(w)) bad = true;
         if (s >= own_lo && s < own_hi) km = key_max(km, mag_key(w));
         Lx[lb + t] = w / xp;
+        if (slots) d.Ls[lb + t] = s;
     }
     km = warp_max_key(km);
     const V amax = key_value<V>(km);

@@ -230,3 +230,16 @@ void bk_launch_levels(const bk_dev &d, int32_t epoch, long long budget, int bloc
     bk_level_scan<<<1, 1024, 0, s>>>(cnt, d.n + 1, stale);
     bk_level_scatter<<<g, 256, 0, s>>>(d.level, d.n, cnt, d.order, stale);
 }
+
+void bk_launch_order(const bk_dev &d, void *stream)
+{
+    cudaStream_t s = (cudaStream_t)stream;
+    int32_t *cnt = d.level + d.n;
+    int32_t *stale = d.counter + 6;
+    const int g = std::max(1, std::min((d.n + 255) / 256, 152 * 8));
+    cudaMemsetAsync(stale, 0xff, sizeof(int32_t), s);
+    cudaMemsetAsync(cnt, 0, sizeof(int32_t) * ((size_t)d.n + 2), s);
+    bk_level_count<<<g, 256, 0, s>>>(d.level, d.n, cnt, stale);
+    bk_level_scan<<<1, 1024, 0, s>>>(cnt, d.n + 1, stale);
+    bk_level_scatter<<<g, 256, 0, s>>>(d.level, d.n, cnt, d.order, stale);
+}
