@@ -48,7 +48,7 @@ struct basker_s {
     int32_t *h_stage = nullptr;      // pinned, 3n + ntasks + 16 ints
     bk_status *h_status = nullptr;   // pinned
     int32_t *h_task_fail = nullptr;  // pinned
-    int32_t epoch = 0, solve_epoch = 0, refno = 0;
+    int32_t epoch = 0, refno = 0;
     bool factored = false, ws_dirty = false, schedule_valid = true, order_is_symbolic = true;
     bool leaf_levels = false;    // the teams wrote the leaves' column levels (all the solve reads)
     bool order_stale = false;    // the stored claim order does not belong to the stored levels
@@ -496,7 +496,7 @@ int setup_device(basker_t h)
     TRY(dalloc(h, &d.ws, (size_t)std::max<int64_t>(pl.ws_bytes, 256), true));
     TRY(dalloc(h, &d.done, (size_t)n, true));
     TRY(dalloc(h, &d.order, (size_t)n));
-    TRY(dalloc(h, &d.counter, 8, true));
+    TRY(dalloc(h, &d.counter, 16, true));
     TRY(dalloc(h, &d.level, (size_t)n * 2 + 2, true));
     TRY(dalloc(h, &d.ahat, (size_t)pl.ahat_doubles));
     TRY(dalloc(h, &d.abits, (size_t)pl.ahat_words));
@@ -581,6 +581,23 @@ int setup_device(basker_t h)
     TRY(upload(h, (int32_t **)&s.cutlo, h->sp.cutlo));
     TRY(upload(h, (int32_t **)&s.cuthi, h->sp.cuthi));
     s.nleaves = (int32_t)h->sp.leaf_tasks.size();
+    s.tasks = h->sp.tasks;
+    s.coupling = h->sp.coupling;
+    s.njobs_a = (int32_t)h->sp.jobs_a.size();
+    s.njobs_c = (int32_t)h->sp.jobs_c.size();
+    s.tf0 = h->sp.tf0;
+    s.tb0 = h->sp.tb0;
+    s.tnd0 = h->sp.tnd0;
+    s.tmax = h->sp.tmax;
+    if (s.tasks) {
+        TRY(upload(h, (bk_sjob **)&s.jobs_a, h->sp.jobs_a));
+        TRY(upload(h, (bk_sjob **)&s.jobs_c, h->sp.jobs_c));
+        TRY(upload(h, &s.titems, h->sp.titems));
+        TRY(dalloc(h, &s.tcnt, (size_t)n));
+        s.ntitems = (int32_t)h->sp.titems.size();
+        TRY(dalloc(h, &s.trec, (size_t)s.ntitems));
+        TRY(dalloc(h, &s.tent, (size_t)s.ntitems));
+    }
     s.leaf_rows = h->sp.leaf_rows;
     s.leaf_f0 = h->sp.leaf_f0;
     s.leaf_b0 = h->sp.leaf_b0;
@@ -588,8 +605,9 @@ int setup_device(basker_t h)
     TRY(upload(h, (int32_t **)&s.leaf_tasks, h->sp.leaf_tasks));
     TRY(dalloc(h, &s.leaf_bad, std::max<size_t>(h->sp.leaf_tasks.size(), 1)));
     TRY(dalloc(h, &s.lcnt, (size_t)2 * ((size_t)h->sp.leaf_maxrows + 1)));
-    TRY(dalloc(h, &s.fdone, (size_t)n, true));
-    TRY(dalloc(h, &s.bdone, (size_t)n, true));
+    TRY(upload(h, (int32_t **)&s.sepix, h->sp.sepix));
+    s.nsep = h->sp.nsep;
+    TRY(dalloc(h, &s.part, (size_t)2 * 32 * (size_t)s.nsep));
     TRY(dalloc(h, &s.r.Lrp, (size_t)n + 1));
     TRY(dalloc(h, &s.r.Urp, (size_t)n + 1));
     TRY(dalloc(h, &s.r.Ud, (size_t)n));
@@ -1083,7 +1101,7 @@ int capture_finish(basker_t h)
 int finish_factorization(basker_t h, cudaStream_t s)
 {
     if (!h->schedule_valid && !h->leaf_levels) TRY(compute_schedule(h, s));
-    tbeg(h, KT_ROWS, s, 19);
+    tbeg(h, KT_ROWS, s, h->sd.tasks ? 16 + (h->sd.nleaves > 0) : 19);
     if (h->opt.graphs) {
         if (!h->g_finish || h->g_finish_ver != h->arena_ver) TRY(capture_finish(h));
         CU(cudaGraphLaunch(h->g_finish, s));
@@ -1467,10 +1485,8 @@ int solve_refined(basker_t h, int32_t nrhs, const double *b, int32_t ldb, double
     double prev = INFINITY;
     for (int it = 1;; it++) {
         CU(cudaMemsetAsync(zmax, 0, sizeof(double) * 2 * (size_t)nrhs, s));
-        CU(cudaMemsetAsync(h->d.counter + 2, 0, sizeof(int32_t), s));
-        h->solve_epoch++;
-        tbeg(h, KT_SOLVE, s, 1);
-        bk_launch_solve(h->d, h->sd, nrhs, h->ir_r, n, h->ir_dz, n, h->solve_epoch, h->opt.wait_budget_cycles, s,
+        tbeg(h, KT_SOLVE, s, bk_solve_kernels(h->sd, nrhs));
+        bk_launch_solve(h->d, h->sd, nrhs, h->ir_r, n, h->ir_dz, n, h->opt.wait_budget_cycles, s,
                         false, h->tune_solve);
         tend(h, s);
         tbeg(h, KT_REFINE, s, 2);
@@ -1529,10 +1545,8 @@ int bk_solve_on_scratch(basker_t h, int32_t nrhs, const double *b_dev, int32_t l
     sd.w = scratch;
     sd.z = scratch + (size_t)nrhs * (size_t)h->pl.n;
     cudaStream_t s = (cudaStream_t)stream;
-    CU(cudaMemsetAsync(h->d.counter + 2, 0, sizeof(int32_t), s));
-    h->solve_epoch++;
-    h->info.kernel_launches++;
-    bk_launch_solve(h->d, sd, nrhs, b_dev, ldb, x_dev, ldx, h->solve_epoch, h->opt.wait_budget_cycles, s, true,
+    h->info.kernel_launches += bk_solve_kernels(h->sd, nrhs);
+    bk_launch_solve(h->d, sd, nrhs, b_dev, ldb, x_dev, ldx, h->opt.wait_budget_cycles, s, true,
                     h->tune_solve);
     CU(cudaGetLastError());
     return BASKER_OK;
@@ -1685,11 +1699,9 @@ int basker_solve(basker_t h, int32_t nrhs, const double *b_dev, int32_t ldb, dou
     if (h->opt.precision) return solve_refined(h, nrhs, b_dev, ldb, x_dev, ldx, (cudaStream_t)stream);
     TRY(ensure_solve_buffers(h, nrhs));
     cudaStream_t s = (cudaStream_t)stream;
-    CU(cudaMemsetAsync(h->d.counter + 2, 0, sizeof(int32_t), s));
-    h->solve_epoch++;
     h->info.precision_used = 0;
-    tbeg(h, KT_SOLVE, s, 1);
-    bk_launch_solve(h->d, h->sd, nrhs, b_dev, ldb, x_dev, ldx, h->solve_epoch, h->opt.wait_budget_cycles, s, true,
+    tbeg(h, KT_SOLVE, s, bk_solve_kernels(h->sd, nrhs));
+    bk_launch_solve(h->d, h->sd, nrhs, b_dev, ldb, x_dev, ldx, h->opt.wait_budget_cycles, s, true,
                     h->tune_solve);
     tend(h, s);
     CU(cudaGetLastError());

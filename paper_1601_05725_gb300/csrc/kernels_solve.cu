@@ -8,10 +8,16 @@
 //   forward row i   w_i = c(prow i) - sum_k L(i,k) w_k, k ascending, after the
 //                   coupling terms of row prow i (later blocks' final z_j)
 //   backward row i  z_i = (w_i - sum_k U(i,k) z_k) / U(i,i), k descending
-// Each term waits for the flag of the row it reads (point-to-point
-// synchronisation, Sec. IV) with a bounded wait.  Per solution entry the fma
+// Each term waits for the value it reads (point-to-point synchronisation, Sec.
+// IV) with a bounded wait.  Per solution entry the fma
 // sequence is the one of the column sweeps (ascending steps for L, descending for
 // U), so the result does not depend on the schedule.
+//
+// What bounds it: the chains of rows, and a row's serial chain of fmas (about 70
+// cycles a term with the next batch's values and terms on their way; 165 when each
+// batch waited for its flags, its values and its terms in turn).  The 316 x 316
+// grid's solve 2.1 ms, was 3.0; eight right-hand sides, a lane each, 3.4 ms, was 67
+// when they ran one after the other through the same chains.
 //
 // The factors are kept by columns; after every factorization bk_launch_rows
 // transposes them into rows (count, scan, scatter, and a rank sort per row).
@@ -23,6 +29,7 @@
 #include "basker_internal.h"
 #include "device_util.cuh"
 #include "solve_internal.h"
+#include "solve_word.cuh"
 #include "trace.cuh"
 
 using namespace bk;
@@ -338,86 +345,151 @@ __global__ void bk_leaf_scatter(bk_dev d, bk_solve_dev s, int chunks)
 
 // ---------------------------------------------------------------- the solve
 
-// One lane's bounded wait until *flag == epoch (an acquiring load, which orders
-// the lane's later reads), sleeping between polls.  False if the wait ran out
-// (the timeout status is then set).
-__device__ __forceinline__ bool poll_flag(const bk_dev &d, const int32_t *flag, int epoch, long long budget)
+// A value that is not final yet is a word of ones (solve_word.cuh): a reader polls
+// the value itself, so a link of the dataflow is one access, without flag or fence.
+
+// One lane's bounded wait for the value at p, sleeping between polls.  The word of
+// ones again if the wait ran out (the timeout status is then set).
+template <typename V>
+__device__ __forceinline__ typename SvWord<V>::U await_value(const bk_dev &d, const typename SvWord<V>::U *p,
+                                                             long long budget)
 {
+    typedef SvWord<V> SW;
+    typename SW::U v = SW::load(p);
+    if (v != SW::none) return v;
     const long long t0 = clock64();
     unsigned ns = 32;
-    while (ld_acquire(flag) != epoch) {
+    while ((v = SW::load(p)) == SW::none) {
         if (*reinterpret_cast<const volatile int *>(&d.status->timeout) || clock64() - t0 > budget) {
             atomicExch(&d.status->timeout, 1);
-            return false;
+            return SW::none;
         }
         __nanosleep(ns);
         ns = min(ns * 2, 128u);
     }
+    return v;
+}
+
+// z -= sum over the terms [e0, e1) of a row, a_e * v(k_e), in their order, one
+// right-hand side (every lane computes the same chain): 32 terms a batch, a lane
+// each; the next batch's values and the one after's terms are read while a batch is
+// applied.  Terms are applied as soon as every earlier one is there; the first
+// missing one is polled by its lane.  The terms end before the first k with
+// (k < cut) != below (cut < 0: at e1).  False if a wait ran out.
+template <typename V>
+__device__ __forceinline__ bool row_terms(const bk_dev &d, const typename SvWord<V>::U *src, const int32_t *rk,
+                                          const int32_t *pos, const V *rx, int64_t e0, int64_t e1, int cut, bool below,
+                                          long long budget, V &z)
+{
+    typedef SvWord<V> SW;
+    typedef typename SW::U U;
+    const int lane = threadIdx.x & 31;
+    auto read = [&](int64_t e, int &k, V &a) {
+        const bool in = e + lane < e1;
+        k = in ? rk[e + lane] : -1;
+        a = in ? rx[pos ? (int64_t)pos[e + lane] : e + lane] : V(0);
+        if (cut >= 0 && k >= 0 && (k < cut) != below) k = -1;
+    };
+    int k, k1, k2;
+    V a, a1, a2;
+    read(e0, k, a);
+    read(e0 + 32, k1, a1);
+    U v = k >= 0 ? SW::load(src + k) : U(0);
+    for (int64_t e = e0; e < e1; e += 32) {
+        const int cnt = __popc(__ballot_sync(BK_FULL, k >= 0));
+        if (cnt == 0) return true;
+        const U v1 = k1 >= 0 ? SW::load(src + k1) : U(0);
+        read(e + 64, k2, a2);
+        for (int done = 0;;) {
+            const uint32_t nr = __ballot_sync(BK_FULL, k >= 0 && v == SW::none);
+            const int upto = nr ? __ffs(nr) - 1 : cnt;
+            const V vv = SW::value(v);
+            int t = done;
+            for (; t + 4 <= upto; t += 4) {
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    z = fma(-__shfl_sync(BK_FULL, a, t + u), __shfl_sync(BK_FULL, vv, t + u), z);
+            }
+            for (; t < upto; t++) z = fma(-__shfl_sync(BK_FULL, a, t), __shfl_sync(BK_FULL, vv, t), z);
+            if (upto >= cnt) break;
+            done = upto;
+            if (v == SW::none && k >= 0) v = lane == done ? await_value<V>(d, src + k, budget) : SW::load(src + k);
+            if (__shfl_sync(BK_FULL, v == SW::none, done)) return false;
+        }
+        if (cnt < 32) return true;
+        k = k1;
+        a = a1;
+        v = v1;
+        k1 = k2;
+        a1 = a2;
+    }
     return true;
 }
 
-// Bounded wait until flags[j] == epoch for every lane with want.  Each lane
-// checks its flag once; lane 0 alone then polls the flags still unset, in lane
-// order (one poller per warp, and no rereads of the other flags meanwhile), and
-// finally each of those lanes rereads its own flag with an acquiring load, which
-// orders its later reads.  False if a wait ran out.
-__device__ __forceinline__ bool wait_flags(const bk_dev &d, const int32_t *flags, int j, bool want, int epoch,
-                                           long long budget)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t pending = __ballot_sync(BK_FULL, want && ld_acquire(flags + j) != epoch);
-    if (!pending) return true;
-    int ok = 1;
-    for (uint32_t p = pending; p; p &= p - 1) {
-        const int jt = __shfl_sync(BK_FULL, j, __ffs(p) - 1);
-        if (lane == 0 && ok) ok = poll_flag(d, flags + jt, epoch, budget);
-    }
-    if (!__shfl_sync(BK_FULL, ok, 0)) return false;
-    int mine = 1;
-    if ((pending >> lane) & 1u) mine = poll_flag(d, flags + j, epoch, budget);
-    return __all_sync(BK_FULL, mine);
-}
-
-// z -= sum over up to 32 terms a_t * v_t, v_t = vals[j_t] once flags[j_t] ==
-// epoch, in lane order (every lane computes the same chain).  The terms whose
-// flags are set are applied as soon as every earlier term is, and the first term
-// still waited for is polled by its own lane: the term that arrives last (in a
-// chain of rows, the previous row) costs one fma after its flag, not a batch.
-// False if a wait ran out (the timeout status is then set).
+// The same for R right-hand sides, the lane's one being q: a batch's terms a lane
+// each, their values eight at a time, the next eight read while eight are applied.
 template <typename V>
-__device__ __forceinline__ bool chain_wait(const bk_dev &d, const int32_t *flags, const V *vals, int j, bool have,
-                                           V a, int cnt, int epoch, long long budget, V &z)
+__device__ __forceinline__ bool row_terms_multi(const bk_dev &d, const typename SvWord<V>::U *src, const int32_t *rk,
+                                                const int32_t *pos, const V *rx, int64_t e0, int64_t e1, int cut,
+                                                bool below, int R, int q, long long budget, V &z)
 {
+    typedef SvWord<V> SW;
+    typedef typename SW::U U;
     const int lane = threadIdx.x & 31;
-    bool ready = !have || ld_acquire(flags + j) == epoch;
-    V v = (have && ready) ? __ldcg(vals + j) : V(0);
-    for (int done = 0;;) {
-        const uint32_t nr = __ballot_sync(BK_FULL, !ready);
-        const int upto = nr ? __ffs(nr) - 1 : cnt;
-        for (int t = done; t < upto; t++) z = fma(-__shfl_sync(BK_FULL, a, t), __shfl_sync(BK_FULL, v, t), z);
-        if (upto >= cnt) return true;
-        done = upto;
-        int ok = 1;
-        if (lane == done) {
-            ok = poll_flag(d, flags + j, epoch, budget);
-            if (ok) {
-                v = __ldcg(vals + j);
-                ready = true;
+    auto read = [&](int64_t e, int &k, V &a) {
+        const bool in = e + lane < e1;
+        k = in ? rk[e + lane] : -1;
+        a = in ? rx[pos ? (int64_t)pos[e + lane] : e + lane] : V(0);
+        if (cut >= 0 && k >= 0 && (k < cut) != below) k = -1;
+    };
+    int k, k1;
+    V a, a1;
+    read(e0, k, a);
+    for (int64_t e = e0; e < e1; e += 32) {
+        const int cnt = __popc(__ballot_sync(BK_FULL, k >= 0));
+        if (cnt == 0) return true;
+        read(e + 32, k1, a1);
+        U v[8], w[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int j = __shfl_sync(BK_FULL, k, u);
+            v[u] = u < cnt ? SW::load(src + (int64_t)j * R + q) : U(0);
+        }
+#pragma unroll
+        for (int t0 = 0; t0 < 32; t0 += 8) {
+            if (t0 >= cnt) break;
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const int t = t0 + 8 + u, j = __shfl_sync(BK_FULL, k, t & 31);
+                w[u] = t < cnt ? SW::load(src + (int64_t)j * R + q) : U(0);
             }
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const int t = t0 + u, j = __shfl_sync(BK_FULL, k, t);
+                const V at = __shfl_sync(BK_FULL, a, t);
+                if (t < cnt) {
+                    if (__any_sync(BK_FULL, v[u] == SW::none)) {
+                        if (v[u] == SW::none) v[u] = await_value<V>(d, src + (int64_t)j * R + q, budget);
+                        if (__any_sync(BK_FULL, v[u] == SW::none)) return false;
+                    }
+                    z = fma(-at, SW::value(v[u]), z);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = w[u];
         }
-        if (!__shfl_sync(BK_FULL, ok, done)) return false;
-        if (!ready && ld_acquire(flags + j) == epoch) {
-            v = __ldcg(vals + j);
-            ready = true;
-        }
+        if (cnt < 32) return true;
+        k = k1;
+        a = a1;
     }
+    return true;
 }
 
 // ---------------------------------------------------------------- separator sweeps
 //
 // One block solves a separator's own triangle, its rows' outside terms already
-// applied (the rows' values in zs, in shared memory or in place in global
-// memory).  Forward: for k ascending, w_k = zs[k] is final and L(i,k) w_k is
+// applied (the rows' values in s.part; in zs, in shared memory or in place in global
+// memory, while they are swept).  Forward: for k ascending, w_k = zs[k] is final and L(i,k) w_k is
 // subtracted from the node's rows i > k; backward: for k descending, z_k =
 // zs[k] / U(k,k) is final and U(j,k) z_k is subtracted from the node's rows
 // j < k.  Per row the terms come in the order of the row sweeps (ascending k
@@ -433,6 +505,7 @@ constexpr int SW_MR = 4 * SW_P;  // ring of column extents
 constexpr int SW_WMAX = 448;   // most entries of a column a stage holds
 constexpr int SW_MAXB = 64;    // most sweeper blocks
 constexpr int SEP_SMEM_ROWS = 1024;   // most rows of a node swept in shared memory
+constexpr int SW_ZMAX = 15 * 1024;    // most values of a node swept in shared memory (rows times right-hand sides)
 
 __host__ __device__ constexpr size_t sw_align(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -476,21 +549,27 @@ __device__ __forceinline__ void sw_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void sw_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename V>
-__device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, int nrhs, double *x, int ldx,
-                                int epoch, long long budget, const int32_t *Qout, unsigned char *smem)
+template <typename V, bool MULTI>
+__device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, int R, double *x, int ldx,
+                                long long budget, const int32_t *Qout, unsigned char *smem)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t n = d.n;
+    const int tid = threadIdx.x;
     const bool fwd = it >= 0;
-    const int t = (fwd ? it : ~it) - (int)n;
+    const int t = (fwd ? it : ~it) - d.n;
+    // right-hand side and entry (of SW_NT / R) of this thread
+    const int rr = MULTI ? R : 1;
+    const int q = MULTI ? tid % rr : 0, g0 = MULTI ? tid / rr : tid, gs = MULTI ? SW_NT / rr : SW_NT;
+    const bool on = g0 < gs;
     const int lo = d.tasks[t].lo, hi = d.tasks[t].hi, m = hi - lo;
+    if (m <= 0) return;
     const int W = s.sw_win;
     const V *const Lx = vals<V>(d.Lx);
     const V *const Ux = vals<V>(d.Ux);
-    V *const w = vals<V>(s.w);
-    V *const zz = vals<V>(s.z);
-    const SwLayout Ly = sw_layout(W, s.sw_zrows, sizeof(V));
+    typedef SvWord<V> SW;
+    typedef typename SW::U U;
+    U *const gout = reinterpret_cast<U *>(vals<V>(fwd ? s.w : s.z)) + (int64_t)lo * rr;
+    U *const part = reinterpret_cast<U *>(vals<V>(s.part)) + ((int64_t)s.sepix[lo] + (fwd ? 0 : s.nsep)) * rr;
+    const SwLayout Ly = sw_layout(W, s.sw_zrows * rr, sizeof(V));
     V *const zsm = reinterpret_cast<V *>(smem);
     int32_t *const ri = reinterpret_cast<int32_t *>(smem + Ly.ri);
     V *const rv = reinterpret_cast<V *>(smem + Ly.rv);
@@ -498,10 +577,13 @@ __device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, 
     int64_t *const mb = reinterpret_cast<int64_t *>(smem + Ly.mb);
     int32_t *const mc = reinterpret_cast<int32_t *>(smem + Ly.mc);
     BK_TSTART(t0);
-    int32_t *flags = fwd ? s.fdone : s.bdone;
+    V *const zs = m <= s.sw_zrows ? zsm : reinterpret_cast<V *>(part);
     bool ok = true;
-    for (int r0 = lo + 32 * warp; r0 < hi && ok; r0 += SW_NT)
-        ok = wait_flags(d, flags, r0 + lane, r0 + lane < hi, -epoch, budget);
+    for (int r = tid; r < m * rr && ok; r += SW_NT) {
+        const U v = await_value<V>(d, part + r, budget);
+        ok = v != SW::none;
+        if (zs == zsm) zs[r] = SW::value(v);
+    }
     if (__syncthreads_or(!ok)) return;
     BK_TPHASE0(tp);
     // the column at sweep position p, and its own entries held by a stage
@@ -522,11 +604,7 @@ __device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, 
         }
         if (!fwd && tid == 0) sw_cpv(rd + st, Ux + beg + cnt - 1);
     };
-    for (int q = 0; q < nrhs; q++) {
-        V *vq = (fwd ? w : zz) + q * n;
-        V *zs = m <= s.sw_zrows ? zsm : vq + lo;
-        if (zs == zsm)
-            for (int r = tid; r < m; r += SW_NT) zs[r] = __ldcg(vq + lo + r);
+    {
         for (int p = tid; p < min(2 * SW_P, m); p += SW_NT) {
             const int c = col_of(p);
             mb[p % SW_MR] = fwd ? d.Lbeg[c] : d.Ubeg[c];
@@ -543,25 +621,29 @@ __device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, 
             sw_wait<SW_P - 2>();
             __syncthreads();
             // the previous step's z (backward) is stored once every thread read it
-            if (kprev >= 0 && tid == 0) zs[kprev] = zprev;
+            if (kprev >= 0 && g0 == 0 && on) zs[kprev * rr + q] = zprev;
             const int kl = fwd ? p : m - 1 - p;
             const int st = p % SW_P, slot = p % SW_MR;
             const int cnt = mc[slot];
             const int64_t beg = mb[slot];
-            V v = zs[kl];
+            V v = zs[kl * rr + q];
             if (!fwd) v = v / rd[st];
             const int wn = own_win(p, cnt);
-            for (int e = tid; e < wn; e += SW_NT) {
+            for (int e = on ? g0 : wn; e < wn; e += gs) {
                 const int r = ri[st * W + e];
-                if (fwd ? r < hi : r >= lo) zs[r - lo] = fma(-rv[st * W + e], v, zs[r - lo]);
+                if (fwd ? r < hi : r >= lo) {
+                    const int at = (r - lo) * rr + q;
+                    zs[at] = fma(-rv[st * W + e], v, zs[at]);
+                }
             }
             // own entries past the stage's window, read directly
             const int own = fwd ? min(cnt, m - 1 - kl) : min(cnt - 1, kl);
-            for (int e = W + tid; e < own; e += SW_NT) {
+            for (int e = on ? W + g0 : own; e < own; e += gs) {
                 const int64_t g = fwd ? beg + e : beg + cnt - 2 - e;
                 const int r = fwd ? s.r.Ls[g] : d.Ui[g];
                 if (fwd ? r >= hi : r < lo) break;
-                zs[r - lo] = fma(-(fwd ? Lx[g] : Ux[g]), v, zs[r - lo]);
+                const int at = (r - lo) * rr + q;
+                zs[at] = fma(-(fwd ? Lx[g] : Ux[g]), v, zs[at]);
             }
             if (!fwd) {
                 zprev = v;
@@ -579,118 +661,96 @@ __device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, 
         }
         sw_wait<0>();
         __syncthreads();
-        if (kprev >= 0 && tid == 0) zs[kprev] = zprev;
+        if (kprev >= 0 && g0 == 0 && on) zs[kprev * rr + q] = zprev;
         __syncthreads();
-        for (int r = tid; r < m; r += SW_NT) {
+        for (int r = tid; r < m * rr; r += SW_NT) {
             const V v = zs[r];
-            vq[lo + r] = v;
-            if (!fwd) x[(int64_t)q * ldx + (Qout ? Qout[lo + r] : lo + r)] = (double)v;
+            U vb = SW::bits(v);
+            if (vb == SW::none) vb = SW::plain_nan;
+            SW::store(gout + r, vb);
+            if (!fwd) {
+                const int row = lo + r / rr;
+                x[(int64_t)(r % rr) * ldx + (Qout ? Qout[row] : row)] = (double)v;
+            }
         }
         __syncthreads();
     }
-    __threadfence();
-    __syncthreads();
-    for (int r = lo + tid; r < hi; r += SW_NT) st_release(flags + r, epoch);
     if (tid == 0) BK_TREC(d.trace, BK_TR_SOLVE, fwd ? 2 : 3, t, t0);
     BK_TPHASE(d.trace, tp, fwd ? 10 : 11, t);     // the sweep itself
 }
 
-template <typename V>
-__global__ void __launch_bounds__(128) bk_solve_kernel(bk_dev d, bk_solve_dev s, int32_t nrhs,
+// MULTI: R right-hand sides, one a lane (R <= 32); else one.  w and z hold row i's
+// values at [i * R, (i + 1) * R).
+template <typename V, bool MULTI>
+__global__ void __launch_bounds__(128) bk_solve_kernel(bk_dev d, bk_solve_dev s, int32_t R,
                                                        const double *__restrict__ b, int32_t ldb, double *x,
-                                                       int32_t ldx, int32_t epoch, long long budget,
+                                                       int32_t ldx, long long budget, int32_t *counter,
                                                        const int32_t *__restrict__ Pin,
                                                        const int32_t *__restrict__ Qout)
 {
+    typedef SvWord<V> SW;
+    typedef typename SW::U U;
     extern __shared__ __align__(16) double solve_smem[];
     const int lane = threadIdx.x & 31;
-    const int64_t n = d.n;
     // the first blocks sweep the separators' own triangles, in claim order
     const int nsb = min(s.nsweeps, SW_MAXB);
     if ((int)blockIdx.x < nsb) {
         for (int k = blockIdx.x; k < s.nsweeps; k += nsb) {
-            sep_sweep_block<V>(d, s, s.sweeps[k], nrhs, x, ldx, epoch, budget, Qout,
-                               reinterpret_cast<unsigned char *>(solve_smem));
+            sep_sweep_block<V, MULTI>(d, s, s.sweeps[k], R, x, ldx, budget, Qout,
+                                      reinterpret_cast<unsigned char *>(solve_smem));
             if (__syncthreads_or(*reinterpret_cast<const volatile int *>(&d.status->timeout) != 0)) return;
         }
         return;
     }
     const V *const Bx = vals<V>(d.Bx);
-    const V *const Lrx = vals<V>(s.r.Lrx);
-    const V *const Urx = vals<V>(s.r.Urx);
     const V *const Ud = vals<V>(s.r.Ud);
-    V *const w = vals<V>(s.w);
-    V *const zz = vals<V>(s.z);
+    U *const gw = reinterpret_cast<U *>(vals<V>(s.w));
+    U *const gz = reinterpret_cast<U *>(vals<V>(s.z));
+    U *const part = reinterpret_cast<U *>(vals<V>(s.part));
+    const int rr = MULTI ? R : 1, q = MULTI ? min(lane, rr - 1) : 0;
+    auto terms = [&](const U *src, const int32_t *rk, const int32_t *pos, const V *rx, int64_t e0, int64_t e1, int cut,
+                     bool below, V &z) {
+        return MULTI ? row_terms_multi<V>(d, src, rk, pos, rx, e0, e1, cut, below, rr, q, budget, z)
+                     : row_terms<V>(d, src, rk, pos, rx, e0, e1, cut, below, budget, z);
+    };
     for (;;) {
         int k = 0;
-        if (lane == 0) k = atomicAdd(d.counter + 2, 1);
+        if (lane == 0) k = atomicAdd(counter, 1);
         k = __shfl_sync(BK_FULL, k, 0);
         if (k >= s.nitems) break;
         const int it = s.items[k];
         BK_TSTART(t0);
         const bool fwd = it >= 0;
         const int i = fwd ? it : ~it;
-        if (i >= n) continue;     // a separator's sweep (the sweeper blocks take it)
+        if (i >= d.n) continue;   // a separator's sweep (the sweeper blocks take it)
         // a separator's row takes only the terms from outside its node
-        const int clo = s.cutlo[i], chi = s.cuthi[i];
-        const bool part = clo >= 0;
+        const int px = s.sepix[i];
+        V z;
         if (fwd) {
-            // forward row i: coupling terms of row prow i, then L(i,k) for k < clo (or all)
+            // forward row i: coupling terms of row prow i, then L(i,k) for k below the node (or all)
             const int r = d.prow[i];
-            const int e0 = s.offp[r], e1 = s.offp[r + 1];
             const int64_t l0 = s.r.Lrp[i], l1 = s.r.Lrp[i + 1];
-            for (int q = 0; q < nrhs; q++) {
-                V z = (V)b[(int64_t)q * ldb + (Pin ? Pin[r] : r)];
-                for (int e = e0; e < e1; e += 32) {
-                    const int cnt = min(32, e1 - e);
-                    const bool have = lane < cnt;
-                    const int j = have ? s.offj[e + lane] : 0;
-                    const V a = have ? Bx[s.offpos[e + lane]] : V(0);
-                    if (!chain_wait(d, s.bdone, zz + q * n, j, have, a, cnt, epoch, budget, z)) return;
-                }
-                for (int64_t e = l0; e < l1; e += 32) {
-                    int cnt = (int)min((int64_t)32, l1 - e);
-                    const int j0 = lane < cnt ? s.r.Lrk[e + lane] : 0;
-                    if (part) cnt = __popc(__ballot_sync(BK_FULL, lane < cnt && j0 < clo));
-                    const bool have = lane < cnt;
-                    const int j = have ? j0 : 0;
-                    const V a = have ? Lrx[e + lane] : V(0);
-                    if (!chain_wait(d, s.fdone, w + q * n, j, have, a, cnt, epoch, budget, z)) return;
-                    if (cnt < 32) break;
-                }
-                if (lane == 0) w[q * n + i] = z;
-            }
-            // lane 0 alone wrote what the flag publishes: its release store orders it
-            __syncwarp();
-            if (lane == 0) st_release(s.fdone + i, part ? -epoch : epoch);
-            if (lane == 0) BK_TREC(d.trace, BK_TR_SOLVE, 0, i, t0);
+            z = (V)b[(int64_t)q * ldb + (Pin ? Pin[r] : r)];
+            if (s.coupling && !terms(gz, s.offj, s.offpos, Bx, s.offp[r], s.offp[r + 1], -1, false, z)) return;
+            if (!terms(gw, s.r.Lrk, nullptr, vals<V>(s.r.Lrx), l0, l1, px >= 0 ? s.cutlo[i] : -1, true, z)) return;
         } else {
-            // backward row i: its forward result, then U(i,k) for k >= chi (or all), then the diagonal
-            if (!wait_flags(d, s.fdone, i, lane == 0, epoch, budget)) return;
+            // backward row i: its forward result, then U(i,k) for k above the node (or all), then the diagonal
             const int64_t u0 = s.r.Urp[i], u1 = s.r.Urp[i + 1];
             const V ud = Ud[i];
-            for (int q = 0; q < nrhs; q++) {
-                V z = __shfl_sync(BK_FULL, lane == 0 ? __ldcg(w + q * n + i) : V(0), 0);
-                for (int64_t e = u0; e < u1; e += 32) {
-                    int cnt = (int)min((int64_t)32, u1 - e);
-                    const int j0 = lane < cnt ? s.r.Urk[e + lane] : 0;
-                    if (part) cnt = __popc(__ballot_sync(BK_FULL, lane < cnt && j0 >= chi));
-                    const bool have = lane < cnt;
-                    const int j = have ? j0 : 0;
-                    const V a = have ? Urx[e + lane] : V(0);
-                    if (!chain_wait(d, s.bdone, zz + q * n, j, have, a, cnt, epoch, budget, z)) return;
-                    if (cnt < 32) break;
-                }
-                if (!part) z = z / ud;
-                if (lane == 0) {
-                    zz[q * n + i] = z;
-                    if (!part) x[(int64_t)q * ldx + (Qout ? Qout[i] : i)] = (double)z;
-                }
-            }
-            __syncwarp();
-            if (lane == 0) st_release(s.bdone + i, part ? -epoch : epoch);
-            if (lane == 0) BK_TREC(d.trace, BK_TR_SOLVE, 1, i, t0);
+            const U w = await_value<V>(d, gw + (int64_t)i * rr + q, budget);
+            if (__any_sync(BK_FULL, w == SW::none)) return;
+            z = SW::value(w);
+            if (!terms(gz, s.r.Urk, nullptr, vals<V>(s.r.Urx), u0, u1, px >= 0 ? s.cuthi[i] : -1, false, z)) return;
+            if (px < 0) z = z / ud;
         }
+        U zb = SW::bits(z);
+        if (zb == SW::none) zb = SW::plain_nan;
+        if (MULTI ? lane < rr : lane == 0) {
+            U *const to = px >= 0 ? part + ((int64_t)px + (fwd ? 0 : s.nsep)) * rr : (fwd ? gw : gz) + (int64_t)i * rr;
+            SW::store(to + q, zb);
+            if (!fwd && px < 0) x[(int64_t)q * ldx + (Qout ? Qout[i] : i)] = (double)z;
+        }
+        if (lane == 0) BK_TREC(d.trace, BK_TR_SOLVE, fwd ? 0 : 1, i, t0);
     }
 }
 
@@ -703,7 +763,7 @@ int bk_solve_blocks()
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bk_solve_kernel<double>, 128,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bk_solve_kernel<double, false>, 128,
                                                       4 * SEP_SMEM_ROWS * sizeof(double));
         return std::max(1, sms) * std::max(1, std::min(per, 8));
     }();
@@ -722,14 +782,16 @@ void bk_solve_sweep_setup(bk_solve_dev &s, int32_t sw_maxm)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // the function attribute is shared by every handle: the largest layout, once
     static const bool raised = [] {
-        const int most = (int)sw_layout(SW_WMAX, SEP_SMEM_ROWS, sizeof(double)).total;
-        cudaFuncSetAttribute(bk_solve_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        cudaFuncSetAttribute(bk_solve_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        const int most = (int)sw_layout(SW_WMAX, SW_ZMAX, sizeof(double)).total;
+        cudaFuncSetAttribute(bk_solve_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(bk_solve_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(bk_solve_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(bk_solve_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         return true;
     }();
     (void)raised;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], bk_solve_kernel<double>, SW_NT, s.sw_smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[1], bk_solve_kernel<float>, SW_NT, s.sw_smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], bk_solve_kernel<double, false>, SW_NT, s.sw_smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[1], bk_solve_kernel<float, false>, SW_NT, s.sw_smem);
     for (int k = 0; k < 2; k++) s.sw_cap[k] = std::max(1, sms) * std::max(1, std::min(per[k], 8));
 }
 
@@ -782,6 +844,10 @@ void bk_launch_rows(const bk_dev &d, const bk_rows &r, void *stream)
 
 void bk_launch_leaf_order(const bk_dev &d, const bk_solve_dev &s, void *stream)
 {
+    if (s.tasks) {
+        bk_launch_torder(d, s, stream);
+        return;
+    }
     if (s.nleaves <= 0) return;
     cudaStream_t st = (cudaStream_t)stream;
     // each leaf's rows over up to 32 blocks of 256 threads
@@ -795,22 +861,72 @@ void bk_launch_leaf_order(const bk_dev &d, const bk_solve_dev &s, void *stream)
     bk_leaf_scatter<<<grid, 256, 0, st>>>(d, s, chunks);
 }
 
-void bk_launch_solve(const bk_dev &d, const bk_solve_dev &s, int32_t nrhs, const double *b, int32_t ldb,
-                     double *x, int32_t ldx, int32_t epoch, long long budget, void *stream, bool permute,
+// Right-hand sides of a batch: a lane each, and every job's values in shared memory.
+static int solve_batch(const bk_solve_dev &s, int32_t nrhs)
+{
+    int r = std::min(nrhs, 32);
+    if (s.tasks) r = std::min<int>(r, std::max(1, (int)(BK_TSOLVE_SMEM / 8 / std::max(s.tmax, 1))));
+    return r;
+}
+
+int bk_solve_kernels(const bk_solve_dev &s, int32_t nrhs)
+{
+    const int r = std::max(1, solve_batch(s, nrhs));
+    const int each = (s.nitems > 0) + (s.tasks ? (s.njobs_a > 0) + (s.njobs_c > 0) : 0);
+    return (nrhs + r - 1) / r * each;
+}
+
+void bk_launch_solve(const bk_dev &d, const bk_solve_dev &s0, int32_t nrhs, const double *b, int32_t ldb,
+                     double *x, int32_t ldx, long long budget, void *stream, bool permute,
                      int max_ctas)
 {
     const int32_t *Pin = permute ? d.P : nullptr, *Qout = permute ? d.Q : nullptr;
-    if (s.nitems <= 0) return;
-    // sweeper blocks first, then the row warps' blocks; every block co-resident
-    const int nsb = std::min(s.nsweeps, SW_MAXB);
-    const int cap = s.sw_cap[d.prec ? 1 : 0];
-    const int limit = max_ctas > 0 ? std::min(max_ctas, cap) : cap;
-    const int ctas = nsb + std::max(1, std::min<int>((s.nitems + 3) / 4, limit - nsb));
-    const size_t smem = s.sw_smem;
-    if (d.prec)
-        bk_solve_kernel<float><<<ctas, SW_NT, smem, (cudaStream_t)stream>>>(d, s, nrhs, b, ldb, x, ldx, epoch, budget, Pin,
-                                                                        Qout);
-    else
-        bk_solve_kernel<double><<<ctas, SW_NT, smem, (cudaStream_t)stream>>>(d, s, nrhs, b, ldb, x, ldx, epoch, budget, Pin,
-                                                                         Qout);
+    cudaStream_t st = (cudaStream_t)stream;
+    const int batch = solve_batch(s0, nrhs);
+    int32_t *const counter = d.counter + 8;
+    for (int32_t q0 = 0; q0 < nrhs; q0 += batch) {
+        const int R = std::min(batch, nrhs - q0);
+        bk_solve_dev s = s0;
+        const double *const bq = b + (int64_t)q0 * ldb;
+        double *const xq = x + (int64_t)q0 * ldx;
+        cudaMemsetAsync(counter, 0, 3 * sizeof(int32_t), st);
+        // no value yet (jobs without separators wait for one another only through
+        // the coupling, by their solution)
+        const size_t vs = d.prec ? sizeof(float) : sizeof(double);
+        if (s.nitems > 0) {
+            cudaMemsetAsync(s.w, 0xff, (size_t)d.n * R * vs, st);
+            if (s.nsep > 0) cudaMemsetAsync(s.part, 0xff, (size_t)s.nsep * 2 * R * vs, st);
+        }
+        if (s.nitems > 0 || s.coupling) cudaMemsetAsync(s.z, 0xff, (size_t)d.n * R * vs, st);
+        if (s.tasks)
+            bk_launch_tsolve(d, s, s.jobs_a, s.njobs_a, counter, R, bq, ldb, xq, ldx, budget, permute, stream);
+        if (s.nitems > 0) {
+            // sweeper blocks first, then the row warps' blocks; every block co-resident
+            const int nsb = std::min(s.nsweeps, SW_MAXB);
+            int cap = s.sw_cap[d.prec ? 1 : 0];
+            size_t smem = s.sw_smem;
+            if (R > 1) {
+                s.sw_zrows = std::min(s.sw_zrows, SW_ZMAX / R);
+                smem = sw_layout(s.sw_win, s.sw_zrows * R, sizeof(double)).total;
+                int dev = 0, sms = 0, per = 0;
+                cudaGetDevice(&dev);
+                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+                if (d.prec) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bk_solve_kernel<float, true>, SW_NT, smem);
+                else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bk_solve_kernel<double, true>, SW_NT, smem);
+                cap = std::max(1, sms) * std::max(1, std::min(per, 8));
+            }
+            const int limit = max_ctas > 0 ? std::min(max_ctas, cap) : cap;
+            const int ctas = nsb + std::max(1, std::min<int>((s.nitems + 3) / 4, limit - nsb));
+            if (d.prec) {
+                if (R > 1) bk_solve_kernel<float, true><<<ctas, SW_NT, smem, st>>>(d, s, R, bq, ldb, xq, ldx, budget, counter + 2, Pin, Qout);
+                else bk_solve_kernel<float, false><<<ctas, SW_NT, smem, st>>>(d, s, R, bq, ldb, xq, ldx, budget, counter + 2, Pin, Qout);
+            } else {
+                if (R > 1) bk_solve_kernel<double, true><<<ctas, SW_NT, smem, st>>>(d, s, R, bq, ldb, xq, ldx, budget, counter + 2, Pin, Qout);
+                else bk_solve_kernel<double, false><<<ctas, SW_NT, smem, st>>>(d, s, R, bq, ldb, xq, ldx, budget, counter + 2, Pin, Qout);
+            }
+        }
+        if (s.tasks)
+            bk_launch_tsolve(d, s, s.jobs_c, s.njobs_c, counter + 1, R, bq, ldb, xq, ldx, budget, permute,
+                             stream);
+    }
 }
