@@ -64,6 +64,11 @@ struct basker_s {
     // reach kernel (listed on the device) and the fast kernel's shared memory
     int32_t *df_redo = nullptr;
     std::vector<bk_desc_par> df_par;     // the descendant phase's on-chip sizes per ND level
+    // the reach of separator columns with their descendant nodes in parallel: logs,
+    // shared memory per ND level (0: not on this level), columns it hands on
+    bk_tdesc_dev td{};
+    std::vector<size_t> td_smem;
+    int32_t *td_over = nullptr;
     // the arena as the symbolic pass left it (natural pivots, symbolic pattern and
     // schedule): a factorization first tries the stored-pattern path from it
     int32_t *sym_Li = nullptr, *sym_Ui = nullptr, *sym_n = nullptr;   // sym_n: 8 arrays of n ints
@@ -257,6 +262,7 @@ int alloc_factors(basker_t h)
     TRY(dalloc(h, &r.Ls, (size_t)h->d.lpool_end));
     h->d.Ls = r.Ls;
     TRY(dalloc(h, &r.tx, (size_t)std::max(h->d.lpool_end, h->d.upool_end)));
+    h->td.link = (unsigned long long *)r.tx;
     TRY(dalloc(h, &h->d.Lx, (size_t)h->d.lpool_end + 4));
     TRY(dalloc(h, &h->d.Ui, (size_t)h->d.upool_end));
     TRY(dalloc(h, &h->d.Ux, (size_t)h->d.upool_end));
@@ -296,6 +302,14 @@ int upload_symbolic_pattern(basker_t h)
     CU(cudaMemcpy(h->d.prow, prow.data(), (size_t)pl.n * 4, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(h->d.pinv, pinv.data(), (size_t)pl.n * 4, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(h->d.order, pl.sorder.data(), (size_t)pl.n * 4, cudaMemcpyHostToDevice));
+    // the separator columns' descendant steps (the leading ones of their U pattern)
+    std::vector<int32_t> dc((size_t)pl.n, 0);
+    u = 0;
+    for (int32_t c = 0; c < pl.n; c++) {
+        const bk_task &T = pl.tasks[(size_t)pl.col_task[(size_t)c]];
+        for (int32_t k = 0; k < pl.sUcnt[(size_t)c]; k++) dc[(size_t)c] += pl.sUi[(size_t)u++] < T.lo;
+    }
+    CU(cudaMemcpy(h->d.dcnt, dc.data(), (size_t)pl.n * 4, cudaMemcpyHostToDevice));
     if (!h->d.iorder) TRY(upload(h, (int32_t **)&h->d.iorder, pl.iorder));
     CU(cudaMemcpy(h->d.level, pl.slevel.data(), (size_t)pl.n * 4, cudaMemcpyHostToDevice));
     return BASKER_OK;
@@ -319,6 +333,7 @@ int save_symbolic_image(basker_t h)
     CU(cudaMemcpy(h->sym_Li, d.Li, sizeof(int32_t) * (size_t)pl.lcap, cudaMemcpyDeviceToDevice));
     CU(cudaMemcpy(h->sym_Ui, d.Ui, sizeof(int32_t) * (size_t)pl.ucap, cudaMemcpyDeviceToDevice));
     int32_t *const a[6] = {d.Lcnt, d.Ucnt, d.prow, d.pinv, d.order, d.level};
+    CU(cudaMemcpy(h->sym_n + 7 * n, d.dcnt, n * 4, cudaMemcpyDeviceToDevice));
     for (int i = 0; i < 6; i++) CU(cudaMemcpy(h->sym_n + i * n, a[i], n * 4, cudaMemcpyDeviceToDevice));
     std::vector<int32_t> ident(n);
     for (size_t c = 0; c < n; c++) ident[c] = (int32_t)c;
@@ -337,8 +352,8 @@ int restore_symbolic_image(basker_t h, cudaStream_t s)
     bk_dev &d = h->d;
     CU(cudaMemcpyAsync(d.Li, h->sym_Li, sizeof(int32_t) * (size_t)pl.lcap, cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(d.Ui, h->sym_Ui, sizeof(int32_t) * (size_t)pl.ucap, cudaMemcpyDeviceToDevice, s));
-    int32_t *const a[7] = {d.Lcnt, d.Ucnt, d.prow, d.pinv, d.order, d.level, const_cast<int32_t *>(d.pref)};
-    for (int i = 0; i < 7; i++) CU(cudaMemcpyAsync(a[i], h->sym_n + i * n, n * 4, cudaMemcpyDeviceToDevice, s));
+    int32_t *const a[8] = {d.Lcnt, d.Ucnt, d.prow, d.pinv, d.order, d.level, const_cast<int32_t *>(d.pref), d.dcnt};
+    for (int i = 0; i < 8; i++) CU(cudaMemcpyAsync(a[i], h->sym_n + i * n, n * 4, cudaMemcpyDeviceToDevice, s));
     int64_t *const b[4] = {d.Lbeg, d.Ubeg, d.Lend, d.Uend};
     for (int i = 0; i < 4; i++) CU(cudaMemcpyAsync(b[i], h->sym_beg + i * n, n * 8, cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(d.pool, h->sym_pool, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
@@ -404,6 +419,51 @@ int setup_teams(basker_t h)
     // pass first, on every SM, and the teams only where it rejects pivots.
     h->stored_first = !pl.counts_only && pl.nnz_l_sym + pl.nnz_u_sym >= (int64_t)32 * pl.n;
     h->team_path = !h->team.empty() && (h->sep_dense || !sep) && h->opt.factor_mode == 0;
+    return BASKER_OK;
+}
+
+// The reach of separator columns with their descendant nodes in parallel, where the
+// column's bitmaps fit on chip.
+int setup_tdesc(basker_t h)
+{
+    const bk_plan &pl = h->pl;
+    h->td_smem.assign(pl.level_tasks.size(), 0);
+    if (!h->team_path || pl.level_tasks.size() < 2 || pl.counts_only) return BASKER_OK;
+    // levels with a column of 2,000 steps or more under the natural pivots (supply
+    // rails); fewer steps lie in one or two nodes, and one warp takes them as fast
+    std::vector<char> on(pl.level_tasks.size(), 0);
+    int64_t most = 0;
+    for (size_t l = 1; l < pl.level_tasks.size(); l++) {
+        for (int32_t t : pl.level_tasks[l])
+            for (int32_t c = pl.tasks[(size_t)t].lo; c < pl.tasks[(size_t)t].hi; c++)
+                if (pl.sUcnt[(size_t)c] >= 2000) on[l] = 1;
+        if (on[l]) most = std::max<int64_t>(most, h->lv_ncols[l]);
+    }
+    if (most == 0 || h->stored_first) return BASKER_OK;
+    const int64_t rows = pl.block_ptr[(size_t)pl.nd_block + 1] - pl.block_ptr[(size_t)pl.nd_block];
+    // netlists log some thousand entries a column, a supply rail tied to a fifth of
+    // the rows two to three a row; at most 128 MB in all
+    h->td.cap = (int32_t)(std::min<int64_t>(std::max<int64_t>(4 * rows, 16384), 262144) + 63) & ~63;
+    h->td.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>({most, 304, ((int64_t)128 << 20) / ((int64_t)h->td.cap * 20)}));
+    for (size_t t = 0; t < pl.tasks.size(); t++) {
+        const bk_task &T = pl.tasks[t];
+        if (T.sp_lo < T.lo)
+            h->td.nodes = std::max(h->td.nodes, (int32_t)t - pl.col_task[(size_t)T.sp_lo]);
+    }
+    h->td.nodes = (h->td.nodes + 1) & ~1;
+    if (h->td.nodes > 2048) return BASKER_OK;
+    for (size_t l = 1; l < pl.level_tasks.size(); l++) {
+        size_t sm = 0;
+        for (int32_t t : pl.level_tasks[l]) {
+            const bk_task &T = pl.tasks[(size_t)t];
+            if (T.sp_lo < T.lo) sm = std::max(sm, bk_tdesc_smem(h->td, T.lo - T.sp_lo, (int64_t)T.lo - T.sp_lo + T.lspace));
+        }
+        h->td_smem[l] = on[l] && sm <= BK_TDESC_SMEM ? sm : 0;
+    }
+    TRY(dalloc(h, &h->td.slot, (size_t)h->td.cap * (size_t)h->td.blocks));
+    TRY(dalloc(h, &h->td.l, (size_t)h->td.cap * (size_t)h->td.blocks));
+    TRY(dalloc(h, &h->td.m, (size_t)h->td.cap * (size_t)h->td.blocks));
+    TRY(dalloc(h, &h->td_over, (size_t)pl.n));
     return BASKER_OK;
 }
 
@@ -558,6 +618,7 @@ int setup_device(basker_t h)
         h->lv_ncols[l] = (int32_t)cols.size();
     }
     TRY(setup_teams(h));
+    TRY(setup_tdesc(h));
     TRY(dalloc(h, &h->rd_tasks, (size_t)std::max<size_t>(pl.tasks.size(), 1)));
     TRY(dalloc(h, &h->rd_c0, (size_t)std::max<size_t>(pl.tasks.size(), 1)));
     TRY(dalloc(h, &h->rd_cols, (size_t)std::max(n, 1)));
@@ -750,18 +811,46 @@ int launch_leaves(basker_t h, cudaStream_t s, int pref_mode, bool repair)
 // device), else every column takes the reach.
 int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
 {
+    const int32_t nd0 = h->pl.nd_block >= 0 ? h->pl.block_ptr[(size_t)h->pl.nd_block] : 0;
+    const int32_t nd1 = h->pl.nd_block >= 0 ? h->pl.block_ptr[(size_t)h->pl.nd_block + 1] : 0;
     for (size_t l = 1; l < h->lv_tasks.size(); l++) {
+        if (h->td.slot) {
+            tbeg(h, KT_DESC, s, 1);
+            bk_launch_lsteps(h->d, h->td, nd0, nd1, (int32_t)l - 1, s);
+            CU(cudaGetLastError());
+            tend(h, s);
+            h->launches++;
+        }
         if (h->lv_ncols[l] > 0) {
-            if (stored) {
-                TRY(launch_desc_refactor(h, h->lv_cols[l], h->lv_ncols[l], s, l));
-            } else {
-                CU(cudaMemsetAsync(h->d.counter + 3, 0, sizeof(int32_t), s));
-                tbeg(h, KT_DESC, s, 1);
-                bk_launch_gp_desc(level_dev(h, l), h->lv_cols[l], h->lv_ncols[l], h->d.counter + 3, s);
+            // on the stored patterns; what fails that by the reach, nodes in parallel;
+            // what outgrows its logs by the reach in one warp
+            const bk_dev dl = level_dev(h, l);
+            int32_t *const cnt = h->d.counter;
+            const int32_t *list = h->lv_cols[l], *nlist = nullptr;
+            const int32_t ncols = h->lv_ncols[l];
+            // (a rail's column is 22,000 steps one after the other on its stored pattern:
+            // the reach with its nodes in parallel takes less)
+            const bk_desc_par par = stored && l < h->df_par.size() && !h->td_smem[l] ? h->df_par[l] : bk_desc_par{};
+            CU(cudaMemsetAsync(cnt, 0, 16 * sizeof(int32_t), s));
+            tbeg(h, KT_DESC, s, (par.smem > 0) + (h->td_smem[l] > 0) + 1);
+            if (par.smem) {
+                bk_launch_desc_fast(dl, list, ncols, cnt + 5, h->df_redo, cnt + 7, par, s);
                 CU(cudaGetLastError());
-                tend(h, s);
+                list = h->df_redo;
+                nlist = cnt + 7;
                 h->launches++;
             }
+            if (h->td_smem[l]) {
+                bk_launch_tdesc(dl, h->td, list, ncols, cnt + 11, nlist, h->td_over, cnt + 12, h->td_smem[l], s);
+                CU(cudaGetLastError());
+                list = h->td_over;
+                nlist = cnt + 12;
+                h->launches++;
+            }
+            bk_launch_gp_desc(dl, list, ncols, cnt + 3, s, nlist);
+            CU(cudaGetLastError());
+            tend(h, s);
+            h->launches++;
         }
         for (int g = 0; g < 2; g++) {
             if (h->lv_ndense[g][l] == 0) continue;

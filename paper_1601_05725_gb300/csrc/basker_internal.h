@@ -214,6 +214,23 @@ void bk_launch_levels(const bk_dev &d, int32_t epoch, long long budget, int bloc
 // The claim order from the stored levels alone (levels valid, order not).
 void bk_launch_order(const bk_dev &d, void *stream);
 int bk_static_blocks();
+// kernels_tdesc.cu: the reach of separator columns, the descendant nodes in parallel
+#define BK_TDESC_SMEM (200 * 1024)
+struct bk_tdesc_dev {
+    int32_t *slot = nullptr;         // logs: cap entries a block
+    double *l = nullptr, *m = nullptr;
+    int32_t cap = 0, blocks = 0;
+    int32_t nodes = 0;               // most descendant nodes of a separator
+    // per L entry: where the L column of its row's step lies (start << 20 | length);
+    // an array the factors by rows use later
+    unsigned long long *link = nullptr;
+};
+size_t bk_tdesc_smem(const bk_tdesc_dev &lg, int64_t ndesc, int64_t space);
+// columns whose log does not fit are listed in over[0 .. *nover)
+void bk_launch_tdesc(const bk_dev &d, const bk_tdesc_dev &lg, const int32_t *cols, int32_t ncols, int32_t *counter,
+                     const int32_t *ncols_dev, int32_t *over, int32_t *nover, size_t smem, void *stream);
+// the rows of the L columns of the ND nodes of a level as steps, for it (d.Ls)
+void bk_launch_lsteps(const bk_dev &d, const bk_tdesc_dev &lg, int32_t c0, int32_t c1, int32_t level, void *stream);
 // kernels_team.cu: Algorithm 1 on tasks without descendants, a block of W warps per
 // task, columns in flight together, deciding in order
 #define BK_TEAM_SMEM (220 * 1024)

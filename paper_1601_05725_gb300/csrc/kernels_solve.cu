@@ -426,8 +426,9 @@ __device__ __forceinline__ bool row_terms(const bk_dev &d, const typename SvWord
     return true;
 }
 
-// The same for R right-hand sides, the lane's one being q: a batch's terms a lane
-// each, their values eight at a time, the next eight read while eight are applied.
+// The same for R right-hand sides, the lane's one being q.  Every lane reads every
+// term (the same address over the warp); three groups of eight are under way: one
+// applied, one with its values coming, one with its terms coming.
 template <typename V>
 __device__ __forceinline__ bool row_terms_multi(const bk_dev &d, const typename SvWord<V>::U *src, const int32_t *rk,
                                                 const int32_t *pos, const V *rx, int64_t e0, int64_t e1, int cut,
@@ -435,52 +436,55 @@ __device__ __forceinline__ bool row_terms_multi(const bk_dev &d, const typename 
 {
     typedef SvWord<V> SW;
     typedef typename SW::U U;
-    const int lane = threadIdx.x & 31;
-    auto read = [&](int64_t e, int &k, V &a) {
-        const bool in = e + lane < e1;
-        k = in ? rk[e + lane] : -1;
-        a = in ? rx[pos ? (int64_t)pos[e + lane] : e + lane] : V(0);
-        if (cut >= 0 && k >= 0 && (k < cut) != below) k = -1;
+    constexpr int G = 8;
+    auto read = [&](int64_t e, int (&k)[G], V (&a)[G]) {
+#pragma unroll
+        for (int u = 0; u < G; u++) {
+            const bool in = e + u < e1;
+            k[u] = in ? rk[e + u] : -1;
+            a[u] = in ? rx[pos ? (int64_t)pos[e + u] : e + u] : V(0);
+        }
+        if (cut >= 0)
+#pragma unroll
+            for (int u = 0; u < G; u++)
+                if (k[u] >= 0 && (k[u] < cut) != below) k[u] = -1;
     };
-    int k, k1;
-    V a, a1;
-    read(e0, k, a);
-    for (int64_t e = e0; e < e1; e += 32) {
-        const int cnt = __popc(__ballot_sync(BK_FULL, k >= 0));
-        if (cnt == 0) return true;
-        read(e + 32, k1, a1);
-        U v[8], w[8];
+    auto values = [&](const int (&k)[G], U (&v)[G]) {
 #pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int j = __shfl_sync(BK_FULL, k, u);
-            v[u] = u < cnt ? SW::load(src + (int64_t)j * R + q) : U(0);
+        for (int u = 0; u < G; u++) v[u] = k[u] >= 0 ? SW::load(src + (int64_t)k[u] * R + q) : U(0);
+    };
+    int k0[G], k1[G], k2[G];
+    V a0[G], a1[G], a2[G];
+    U v0[G], v1[G];
+    read(e0, k0, a0);
+    read(e0 + G, k1, a1);
+    values(k0, v0);
+    for (int64_t e = e0; k0[0] >= 0; e += G) {
+        values(k1, v1);
+        read(e + 2 * G, k2, a2);
+        bool miss = false;
+#pragma unroll
+        for (int u = 0; u < G; u++) miss = miss || v0[u] == SW::none;
+        if (__any_sync(BK_FULL, miss)) {
+#pragma unroll
+            for (int u = 0; u < G; u++)
+                if (k0[u] >= 0 && v0[u] == SW::none) v0[u] = await_value<V>(d, src + (int64_t)k0[u] * R + q, budget);
+            miss = false;
+#pragma unroll
+            for (int u = 0; u < G; u++) miss = miss || v0[u] == SW::none;
+            if (__any_sync(BK_FULL, miss)) return false;
         }
 #pragma unroll
-        for (int t0 = 0; t0 < 32; t0 += 8) {
-            if (t0 >= cnt) break;
+        for (int u = 0; u < G; u++)
+            if (k0[u] >= 0) z = fma(-a0[u], SW::value(v0[u]), z);
 #pragma unroll
-            for (int u = 0; u < 8; u++) {
-                const int t = t0 + 8 + u, j = __shfl_sync(BK_FULL, k, t & 31);
-                w[u] = t < cnt ? SW::load(src + (int64_t)j * R + q) : U(0);
-            }
-#pragma unroll
-            for (int u = 0; u < 8; u++) {
-                const int t = t0 + u, j = __shfl_sync(BK_FULL, k, t);
-                const V at = __shfl_sync(BK_FULL, a, t);
-                if (t < cnt) {
-                    if (__any_sync(BK_FULL, v[u] == SW::none)) {
-                        if (v[u] == SW::none) v[u] = await_value<V>(d, src + (int64_t)j * R + q, budget);
-                        if (__any_sync(BK_FULL, v[u] == SW::none)) return false;
-                    }
-                    z = fma(-at, SW::value(v[u]), z);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = w[u];
+        for (int u = 0; u < G; u++) {
+            k0[u] = k1[u];
+            a0[u] = a1[u];
+            v0[u] = v1[u];
+            k1[u] = k2[u];
+            a1[u] = a2[u];
         }
-        if (cnt < 32) return true;
-        k = k1;
-        a = a1;
     }
     return true;
 }

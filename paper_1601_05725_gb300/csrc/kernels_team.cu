@@ -554,10 +554,11 @@ __global__ void __launch_bounds__(512, 1) bk_team_kernel(bk_dev d, const int32_t
                             for (int u = 0; u < TM_PF; u++) {
                                 ss[u] = -1;
                                 ll[u] = V(0);
-                                if (u > 0 && (rl >> 16) <= 32 * u) break;
-                                const int s = rs[lane + 32 * u];
-                                ss[u] = s == 0xffff ? -1 : s;
-                                ll[u] = rv[lane + 32 * u];
+                                if (u == 0 || (rl >> 16) > 32 * u) {
+                                    const int s = rs[lane + 32 * u];
+                                    ss[u] = s == 0xffff ? -1 : s;
+                                    ll[u] = rv[lane + 32 * u];
+                                }
                             }
                             jlev = rl & 0xffff;
                             __syncwarp();
