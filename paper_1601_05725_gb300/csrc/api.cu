@@ -38,11 +38,11 @@ struct basker_s {
     bool stored_first = false;   // the stored-pattern pass before the teams (dense enough columns)
     bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones)
     bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once from then on
-    // separators whose in-node phase runs as one dense elimination, by cluster size
-    // ([0]: one block, [1]: BK_DENSE_CLUSTER blocks)
-    std::vector<int32_t *> lv_dense[2];
-    std::vector<int32_t> lv_ndense[2];
-    std::vector<size_t> lv_dsmem[2];
+    // separators whose in-node phase runs as one dense elimination, by kernel and cluster size
+    // (bk_dense_node_group)
+    std::vector<int32_t *> lv_dense[BK_DENSE_GROUPS];
+    std::vector<int32_t> lv_ndense[BK_DENSE_GROUPS];
+    std::vector<size_t> lv_dsmem[BK_DENSE_GROUPS];
     // redo lists (device buffers of n ints each) and their pinned staging
     int32_t *rd_tasks = nullptr, *rd_c0 = nullptr, *rd_cols = nullptr;
     int32_t *h_stage = nullptr;      // pinned, 3n + ntasks + 16 ints
@@ -584,19 +584,19 @@ int setup_device(basker_t h)
     h->lv_smem.assign(nl, 0);
     h->lv_cols.assign(nl, nullptr);
     h->lv_ncols.assign(nl, 0);
-    for (int g = 0; g < 2; g++) {
+    for (int g = 0; g < BK_DENSE_GROUPS; g++) {
         h->lv_dense[g].assign(nl, nullptr);
         h->lv_ndense[g].assign(nl, 0);
         h->lv_dsmem[g].assign(nl, 0);
     }
     for (size_t l = 0; l < nl; l++) {
-        std::vector<int32_t> ids, dense[2];
-        size_t sm = 0, dsm[2] = {0, 0};
+        std::vector<int32_t> ids, dense[BK_DENSE_GROUPS];
+        size_t sm = 0, dsm[BK_DENSE_GROUPS] = {};
         std::vector<int32_t> cols;
         for (int32_t t : pl.level_tasks[l]) {
             const bk_task &T = pl.tasks[(size_t)t];
             if (h->opt.factor_mode == 0 && bk_dense_node_eligible(T)) {
-                const int g = bk_dense_node_cluster(T) > 1 ? 1 : 0;
+                const int g = bk_dense_node_group(T);
                 dense[g].push_back(t);
                 dsm[g] = std::max(dsm[g], bk_dense_node_smem(T));
             } else {
@@ -608,7 +608,7 @@ int setup_device(basker_t h)
         }
         TRY(upload(h, &h->lv_tasks[l], ids));
         h->lv_ntasks[l] = (int32_t)ids.size();
-        for (int g = 0; g < 2; g++) {
+        for (int g = 0; g < BK_DENSE_GROUPS; g++) {
             TRY(upload(h, &h->lv_dense[g][l], dense[g]));
             h->lv_ndense[g][l] = (int32_t)dense[g].size();
             h->lv_dsmem[g][l] = (dsm[g] + 15) & ~(size_t)15;
@@ -852,11 +852,11 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
             tend(h, s);
             h->launches++;
         }
-        for (int g = 0; g < 2; g++) {
+        for (int g = 0; g < BK_DENSE_GROUPS; g++) {
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], h->opt.tau, pref_mode,
-                                  g ? BK_DENSE_CLUSTER : 1, s);
+                                  g, s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;
@@ -888,11 +888,11 @@ int launch_full_gp(basker_t h, cudaStream_t s, int pref_mode)
             tend(h, s);
             h->launches++;
         }
-        for (int g = 0; g < 2; g++) {
+        for (int g = 0; g < BK_DENSE_GROUPS; g++) {
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], tau, pref_mode,
-                                  g ? BK_DENSE_CLUSTER : 1, s);
+                                  g, s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;
@@ -971,12 +971,12 @@ int launch_redo(basker_t h, cudaStream_t s)
             // instead of rounds of column-by-column recomputation.  All or none:
             // the rounds of a separator rely on the change markers that rounds
             // leave on the columns below it, which the dense path does not set.
-            std::vector<int32_t> dense[2], rest, cols;
-            size_t dsm[2] = {0, 0};
+            std::vector<int32_t> dense[BK_DENSE_GROUPS], rest, cols;
+            size_t dsm[BK_DENSE_GROUPS] = {};
             for (int32_t t : active) {
                 const bk_task &T = pl.tasks[(size_t)t];
                 if (bk_dense_node_eligible(T)) {
-                    const int g = bk_dense_node_cluster(T) > 1 ? 1 : 0;
+                    const int g = bk_dense_node_group(T);
                     dense[g].push_back(t);
                     dsm[g] = std::max(dsm[g], bk_dense_node_smem(T));
                     for (int32_t c = T.lo; c < T.hi; c++) cols.push_back(c);
@@ -987,14 +987,17 @@ int launch_redo(basker_t h, cudaStream_t s)
             if (!cols.empty()) {
                 CU(cudaStreamSynchronize(s));       // the staging buffer is reused
                 TRY(stage_upload(h, s, h->rd_cols, cols, 0));
-                TRY(stage_upload(h, s, h->rd_tasks, dense[0], (size_t)pl.n));
-                TRY(stage_upload(h, s, h->rd_tasks + dense[0].size(), dense[1], (size_t)pl.n + dense[0].size()));
+                size_t at[BK_DENSE_GROUPS + 1] = {};
+                for (int g = 0; g < BK_DENSE_GROUPS; g++) {
+                    at[g + 1] = at[g] + dense[g].size();
+                    TRY(stage_upload(h, s, h->rd_tasks + at[g], dense[g], (size_t)pl.n + at[g]));
+                }
                 TRY(launch_desc_refactor(h, h->rd_cols, (int32_t)cols.size(), s, l));
-                for (int g = 0; g < 2; g++) {
+                for (int g = 0; g < BK_DENSE_GROUPS; g++) {
                     if (dense[g].empty()) continue;
                     tbeg(h, KT_DENSE, s, 1);
-                    bk_launch_dense_nodes(h->d, h->rd_tasks + (g ? dense[0].size() : 0), (int32_t)dense[g].size(),
-                                          (dsm[g] + 15) & ~(size_t)15, tau, 1, g ? BK_DENSE_CLUSTER : 1, s);
+                    bk_launch_dense_nodes(h->d, h->rd_tasks + at[g], (int32_t)dense[g].size(),
+                                          (dsm[g] + 15) & ~(size_t)15, tau, 1, g, s);
                     CU(cudaGetLastError());
                     tend(h, s);
                     h->launches++;
@@ -1103,11 +1106,11 @@ int launch_repair_path(basker_t h, cudaStream_t s)
     h->launches++;
     for (size_t l = 1; l < h->lv_tasks.size(); l++) {
         TRY(launch_desc_refactor(h, h->lv_cols[l], h->lv_ncols[l], s, l));
-        for (int g = 0; g < 2; g++) {
+        for (int g = 0; g < BK_DENSE_GROUPS; g++) {
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], h->opt.tau, 1,
-                                  g ? BK_DENSE_CLUSTER : 1, s);
+                                  g, s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;

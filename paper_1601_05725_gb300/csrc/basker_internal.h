@@ -176,12 +176,18 @@ size_t bk_task_smem_bytes(const bk_task &t);
 size_t bk_dense_node_smem(const bk_task &t);
 bool bk_dense_node_eligible(const bk_task &t);
 // separators of at least BK_DENSE_CLUSTER_MIN columns run on a cluster of
-// BK_DENSE_CLUSTER blocks (columns dealt round-robin), smaller ones on one block
+// BK_DENSE_CLUSTER blocks, smaller ones on one block.  bk_dense_node_group: 0 rows in
+// one block, 1 rows dealt over a cluster (kernels_drows.cu), 2 columns dealt over a
+// cluster, in the scratch (kernels_dense.cu)
 #define BK_DENSE_CLUSTER 8
 #define BK_DENSE_CLUSTER_MIN 64
-int bk_dense_node_cluster(const bk_task &t);
+#define BK_DENSE_GROUPS 3
+int bk_dense_node_group(const bk_task &t);
 void bk_launch_dense_nodes(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                           int pref_mode, int cluster, void *stream);
+                           int pref_mode, int group, void *stream);
+size_t bk_dense_rows_smem(const bk_task &t, int cluster);
+void bk_launch_dense_rows(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
+                          int pref_mode, int cluster, void *stream);
 bool bk_task_fits_smem(const bk_task &t);
 
 // kernels (launchers), kernels_*.cu

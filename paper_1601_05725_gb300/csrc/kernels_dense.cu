@@ -1,5 +1,7 @@
 // kernels_dense.cu -- the in-node phase of an ND separator as a dense
-// right-looking elimination, one block of threads per separator.
+// right-looking elimination, its columns dealt over a cluster of thread blocks: the
+// kernel of separators whose rows do not fit the cluster's shared memory (the others:
+// kernels_drows.cu, which takes a quarter to a half less time).
 //
 // After the descendant phase (Algorithm 4's solves with the descendants' L and
 // the reductions into A-hat) every column of separator j is a dense vector over
@@ -70,9 +72,7 @@ __device__ __forceinline__ void cluster_stop(cg::cluster_group &cl, DnShared &S,
     for (unsigned r = 0; r < cl.num_blocks(); r++) *cl.map_shared_rank(&S.stop[parity], r) = 1;
 }
 
-// Shared memory of a block, in bytes: the base layout, and the block's own
-// columns of the dense block with their pattern words (columns k with
-// k mod cluster == rank), kept on chip when they fit.
+// Shared memory of a block, in bytes.
 __host__ __device__ inline size_t dn_base_bytes(int own, int lsp)
 {
     const size_t nrw = ((size_t)lsp + 31) / 32;
@@ -80,15 +80,9 @@ __host__ __device__ inline size_t dn_base_bytes(int own, int lsp)
            (4 * nrw + 1) * 4 + 2 * (size_t)own + 16;
 }
 
-__host__ __device__ inline size_t dn_local_bytes(int own, int lsp, int cluster)
-{
-    const size_t nloc = ((size_t)own + cluster - 1) / cluster, nrw = ((size_t)lsp + 31) / 32;
-    return nloc * (size_t)lsp * 8 + nloc * nrw * 4;
-}
-
 template <typename V>
 __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, const int32_t *__restrict__ task_ids,
-                                                                   double tau, int pref_mode, size_t smem_bytes)
+                                                                   double tau, int pref_mode)
 {
     V *const Lx = vals<V>(d.Lx);
     V *const Ux = vals<V>(d.Ux);
@@ -106,12 +100,9 @@ __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, con
     __syncthreads();
     const bk_task &T = S.T;
     const int nown = T.hi - T.lo, lsp = T.lspace, nrw = (lsp + 31) >> 5;
-    // the block's columns on chip when they fit in the shared memory given
-    const bool onchip = dn_base_bytes(nown, lsp) + dn_local_bytes(nown, lsp, CN) <= smem_bytes;
-    const int nloc = onchip ? (nown + CN - 1) / CN : 0;
     // shared layout (8-byte slots first): ub[nown] ue[nown] (int64) | lval[2][lsp] colv[lsp]
-    // mval[nown] loc[nloc][lsp] (V in 8-byte slots) | nus[nown] spiv[nown] lsl[2][lsp] wpre[nrw + 1]
-    // lbits[2][nrw] colb[nrw] locb[nloc][nrw] (32-bit) | cbad[nown] chit[nown] (bytes).
+    // mval[nown] (V in 8-byte slots) | nus[nown] spiv[nown] lsl[2][lsp] wpre[nrw + 1]
+    // lbits[2][nrw] colb[nrw] (32-bit) | cbad[nown] chit[nown] (bytes).
     // Per-column state is kept by the block that owns the column (column k: block
     // k mod CN, local index k / CN); spiv by every block.
     int64_t *ubs = reinterpret_cast<int64_t *>(dsm);
@@ -121,8 +112,7 @@ __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, con
     V *lval1 = reinterpret_cast<V *>(slots + lsp);
     V *colv = reinterpret_cast<V *>(slots + 2 * lsp);
     V *mval = reinterpret_cast<V *>(slots + 3 * lsp);
-    double *locslots = slots + 3 * lsp + nown;
-    int32_t *nus = reinterpret_cast<int32_t *>(locslots + (int64_t)nloc * lsp);
+    int32_t *nus = reinterpret_cast<int32_t *>(slots + 3 * lsp + nown);
     int32_t *spiv = nus + nown;
     int32_t *lsl0 = spiv + nown;
     int32_t *lsl1 = lsl0 + lsp;
@@ -130,17 +120,13 @@ __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, con
     uint32_t *lbits0 = reinterpret_cast<uint32_t *>(wpre + nrw + 1);
     uint32_t *lbits1 = lbits0 + nrw;
     uint32_t *colb = lbits1 + nrw;
-    uint32_t *locb = colb + nrw;
-    unsigned char *cbad = reinterpret_cast<unsigned char *>(locb + (int64_t)nloc * nrw);
+    unsigned char *cbad = reinterpret_cast<unsigned char *>(colb + nrw);
     unsigned char *chit = cbad + nown;
 
     V *const A = Ahat + T.ahoff;                       // column k at A + k * lsp
     uint32_t *const AB = d.abits + T.aboff;            // column k at AB + k * nrw
-    // column k of this block (values, pattern words): on chip or in the scratch
-    auto colA = [&](int k) -> V * {
-        return onchip ? reinterpret_cast<V *>(locslots + (int64_t)(k / CN) * lsp) : A + (int64_t)k * lsp;
-    };
-    auto colB = [&](int k) -> uint32_t * { return onchip ? locb + (int64_t)(k / CN) * nrw : AB + (int64_t)k * nrw; };
+    auto colA = [&](int k) -> V * { return A + (int64_t)k * lsp; };
+    auto colB = [&](int k) -> uint32_t * { return AB + (int64_t)k * nrw; };
     for (int k = tid_x; k < nown; k += DN_THREADS) {
         const int c = T.lo + k;
         if (k % CN == rank) {
@@ -157,14 +143,8 @@ __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, con
         const int k = (int)(e / lsp), sl = (int)(e % lsp);
         if (k % CN != rank) continue;
         const bool in = (AB[(int64_t)k * nrw + (sl >> 5)] >> (sl & 31)) & 1u;
-        if (onchip) colA(k)[sl] = in ? A[e] : V(0);
-        else if (!in) A[e] = V(0);
+        if (!in) A[e] = V(0);
     }
-    if (onchip)
-        for (int64_t e = tid_x; e < (int64_t)nown * nrw; e += DN_THREADS) {
-            const int k = (int)(e / nrw);
-            if (k % CN == rank) colB(k)[e % nrw] = AB[e];
-        }
     cl.sync();
 
 #ifdef BK_TRACE
@@ -463,12 +443,19 @@ __global__ void __launch_bounds__(DN_THREADS) bk_dense_node_kernel(bk_dev d, con
 
 }  // namespace
 
+// Rows dealt over the blocks where they fit their shared memory: one block for a node
+// of fewer than BK_DENSE_CLUSTER_MIN columns, else a cluster; columns dealt over a
+// cluster, in the scratch, for a larger node (about 190,000 entries and more).
+int bk_dense_node_group(const bk_task &T)
+{
+    if (T.hi - T.lo < BK_DENSE_CLUSTER_MIN && bk_dense_rows_smem(T, 1) <= BK_DENSE_SMEM) return 0;
+    return bk_dense_rows_smem(T, BK_DENSE_CLUSTER) <= BK_DENSE_SMEM ? 1 : 2;
+}
+
 size_t bk_dense_node_smem(const bk_task &T)
 {
-    const int own = T.hi - T.lo;
-    const size_t base = dn_base_bytes(own, T.lspace);
-    const size_t full = base + dn_local_bytes(own, T.lspace, bk_dense_node_cluster(T));
-    return full <= BK_DENSE_SMEM ? full : base;
+    const int g = bk_dense_node_group(T);
+    return g < 2 ? bk_dense_rows_smem(T, g ? BK_DENSE_CLUSTER : 1) : dn_base_bytes(T.hi - T.lo, T.lspace);
 }
 
 bool bk_dense_node_eligible(const bk_task &T)
@@ -477,9 +464,14 @@ bool bk_dense_node_eligible(const bk_task &T)
 }
 
 void bk_launch_dense_nodes(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                           int pref_mode, int cluster, void *stream)
+                           int pref_mode, int group, void *stream)
 {
     if (ntasks <= 0) return;
+    if (group < 2) {
+        bk_launch_dense_rows(d, task_ids, ntasks, smem, tau, pref_mode, group ? BK_DENSE_CLUSTER : 1, stream);
+        return;
+    }
+    const int cluster = BK_DENSE_CLUSTER;
     static std::once_flag once;
     std::call_once(once, [] {
         cudaFuncSetAttribute(bk_dense_node_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, BK_DENSE_SMEM);
@@ -498,12 +490,7 @@ void bk_launch_dense_nodes(const bk_dev &d, const int32_t *task_ids, int32_t nta
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (d.prec)
-        cudaLaunchKernelEx(&cfg, bk_dense_node_kernel<float>, d, task_ids, tau, pref_mode, smem);
+        cudaLaunchKernelEx(&cfg, bk_dense_node_kernel<float>, d, task_ids, tau, pref_mode);
     else
-        cudaLaunchKernelEx(&cfg, bk_dense_node_kernel<double>, d, task_ids, tau, pref_mode, smem);
-}
-
-int bk_dense_node_cluster(const bk_task &T)
-{
-    return T.hi - T.lo >= BK_DENSE_CLUSTER_MIN ? BK_DENSE_CLUSTER : 1;
+        cudaLaunchKernelEx(&cfg, bk_dense_node_kernel<double>, d, task_ids, tau, pref_mode);
 }
