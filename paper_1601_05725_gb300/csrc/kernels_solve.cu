@@ -140,7 +140,7 @@ __global__ void bk_rows_scatter(bk_dev d, bk_rows r, int which)
             const int64_t lb = d.Lbeg[c];
             const int ln = d.Lcnt[c];
             for (int t = lane; t < ln; t += 32) {
-                const int i = d.pinv[d.Li[lb + t]];
+                const int i = r.Ls[lb + t];             // bk_rows_count
                 const int64_t pos = rp[i] + atomicAdd(cur + i, 1);
                 r.tk[pos] = c;
                 vals<V>(r.tx)[pos] = vals<V>(d.Lx)[lb + t];
@@ -159,35 +159,117 @@ __global__ void bk_rows_scatter(bk_dev d, bk_rows r, int which)
 }
 
 // Each row's entries in ascending (L) or descending (U) column order: the rank of
-// an entry is the number of entries of its row that come before it.
+// an entry is the number of entries of its row that come before it.  A warp a row:
+//   up to 32 entries     compared with each other by shuffles, as many as there are;
+//   up to BK_LONG_ROW    the columns (distinct) set bits of a map in shared memory, over
+//                        the range they span if that is RS_WORDS words at most, else (U)
+//                        over the row's L-space (own columns, then the ancestors'); an
+//                        entry's rank is the set bits before its own.  Linear in the
+//                        row's length and the map;
+//                        else compared with each other, four a shared load.
+// Bound by the instructions of the long rows (a comparison of every pair by shuffles
+// took 256 times 32 for 512 entries).  Measured, L and U: 316 x 316 mesh (3.75 and 3.82
+// million entries) 0.92 -> 0.13 ms, 8192 blocks of up to 1024 rows 1.42 -> 0.44 ms.
+constexpr int RS_WARPS = 8;
+constexpr int RS_WORDS = 512;
+
 template <typename V>
-__global__ void bk_rows_sort(int32_t n, const int64_t *rp, const int32_t *tk, const V *tx, int32_t *ok, V *ox,
-                             int desc)
+__global__ void __launch_bounds__(RS_WARPS * 32) bk_rows_sort(bk_dev d, const int64_t *rp, const int32_t *tk,
+                                                              const V *tx, int32_t *ok, V *ox, int desc)
 {
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    __shared__ __align__(16) int32_t skey[RS_WARPS][BK_LONG_ROW];
+    __shared__ uint32_t sbm[RS_WARPS][RS_WORDS];
+    __shared__ uint16_t spre[RS_WARPS][RS_WORDS];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int warp = blockIdx.x * RS_WARPS + wid;
+    const int nwarps = gridDim.x * RS_WARPS;
     const int sentinel = desc ? INT_MIN : INT_MAX;
-    for (int i = warp; i < n; i += nwarps) {
+    int32_t *const key = skey[wid];
+    uint32_t *const bm = sbm[wid];
+    uint16_t *const pre = spre[wid];
+    for (int i = warp; i < d.n; i += nwarps) {
         const int64_t p0 = rp[i];
         const int len = (int)(rp[i + 1] - p0);
         if (len > BK_LONG_ROW) continue;          // bk_rows_sort_long
-        for (int e0 = 0; e0 < len; e0 += 32) {
-            const bool mine = e0 + lane < len;
-            const int myk = mine ? tk[p0 + e0 + lane] : sentinel;
-            const V myx = mine ? tx[p0 + e0 + lane] : V(0);
+        if (len <= 32) {
+            const bool mine = lane < len;
+            const int myk = mine ? tk[p0 + lane] : sentinel;
+            const V myx = mine ? tx[p0 + lane] : V(0);
             int rank = 0;
-            for (int f0 = 0; f0 < len; f0 += 32) {
-                const int other = f0 + lane < len ? tk[p0 + f0 + lane] : sentinel;
-#pragma unroll 8
-                for (int t = 0; t < 32; t++) {
-                    const int kk = __shfl_sync(BK_FULL, other, t);
+            for (int t = 0; t < len; t += 4)
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int kk = __shfl_sync(BK_FULL, myk, t + u);
                     rank += desc ? (kk > myk) : (kk < myk);
                 }
-            }
             if (mine) {
                 ok[p0 + rank] = myk;
                 ox[p0 + rank] = myx;
+            }
+            continue;
+        }
+        __syncwarp();
+        int lo = INT_MAX, hi = 0;
+        for (int e = lane; e < len; e += 32) {
+            const int c = tk[p0 + e];
+            key[e] = c;
+            lo = min(lo, c);
+            hi = max(hi, c);
+        }
+        lo = __reduce_min_sync(BK_FULL, lo);
+        hi = __reduce_max_sync(BK_FULL, hi);
+        if (((hi - lo) >> 5) >= RS_WORDS && desc) {
+            // over the L-space of the row's task, if all columns are in it
+            const bk_task &T = d.tasks[d.col_task[i]];
+            if (T.lspace <= 32 * RS_WORDS) {
+                bool in = true;
+                for (int e = lane; e < len; e += 32) in = in && slot_of(T, T.lo, key[e]) >= 0;
+                if (__all_sync(BK_FULL, in)) {
+                    for (int e = lane; e < len; e += 32) key[e] = slot_of(T, T.lo, key[e]);
+                    lo = 0;
+                    hi = T.lspace - 1;
+                }
+            }
+        }
+        const int W = ((hi - lo) >> 5) + 1;
+        __syncwarp();
+        if (W <= RS_WORDS) {
+            for (int w = lane; w < W; w += 32) bm[w] = 0u;
+            __syncwarp();
+            for (int e = lane; e < len; e += 32) {
+                const int off = key[e] - lo;
+                atomicOr(bm + (off >> 5), 1u << (off & 31));
+            }
+            __syncwarp();
+            int carry = 0;
+            for (int w0 = 0; w0 < W; w0 += 32) {
+                const int w = w0 + lane;
+                const int n = w < W ? __popc(bm[w]) : 0;
+                const int ex = warp_exscan(n, lane);
+                if (w < W) pre[w] = (uint16_t)(carry + ex);
+                carry += __shfl_sync(BK_FULL, ex + n, 31);
+            }
+            __syncwarp();
+            for (int e = lane; e < len; e += 32) {
+                const int off = key[e] - lo;
+                const int r = pre[off >> 5] + __popc(bm[off >> 5] & ((1u << (off & 31)) - 1u));
+                const int rank = desc ? len - 1 - r : r;
+                ok[p0 + rank] = tk[p0 + e];
+                ox[p0 + rank] = tx[p0 + e];
+            }
+        } else {
+            for (int e = len + lane; e < ((len + 3) & ~3); e += 32) key[e] = sentinel;
+            __syncwarp();
+            for (int e = lane; e < len; e += 32) {
+                const int myk = key[e];
+                int rank = 0;
+                for (int t = 0; t < len; t += 4) {
+                    const int4 o = *reinterpret_cast<const int4 *>(key + t);
+                    rank += desc ? (o.x > myk) + (o.y > myk) + (o.z > myk) + (o.w > myk)
+                                 : (o.x < myk) + (o.y < myk) + (o.z < myk) + (o.w < myk);
+                }
+                ok[p0 + rank] = myk;
+                ox[p0 + rank] = tx[p0 + e];
             }
         }
     }
@@ -834,12 +916,12 @@ void bk_launch_rows(const bk_dev &d, const bk_rows &r, void *stream)
         bk_rows_long_list<<<lblocks, 256, 0, st>>>(n, rp, r.longs);
         if (d.prec) {
             bk_rows_scatter<float><<<blocks, 256, 0, st>>>(d, r, which);
-            bk_rows_sort<float><<<blocks, 256, 0, st>>>(n, rp, r.tk, vals<float>(r.tx), ok, vals<float>(ox), which);
+            bk_rows_sort<float><<<blocks, RS_WARPS * 32, 0, st>>>(d, rp, r.tk, vals<float>(r.tx), ok, vals<float>(ox), which);
             bk_rows_sort_long<float><<<BK_LONG_CTAS, 1024, 0, st>>>(rp, r.tk, vals<float>(r.tx), ok, vals<float>(ox),
                                                                      which, r.longs, r.sbits, r.spre, r.swords);
         } else {
             bk_rows_scatter<double><<<blocks, 256, 0, st>>>(d, r, which);
-            bk_rows_sort<double><<<blocks, 256, 0, st>>>(n, rp, r.tk, r.tx, ok, ox, which);
+            bk_rows_sort<double><<<blocks, RS_WARPS * 32, 0, st>>>(d, rp, r.tk, r.tx, ok, ox, which);
             bk_rows_sort_long<double><<<BK_LONG_CTAS, 1024, 0, st>>>(rp, r.tk, r.tx, ok, ox, which, r.longs, r.sbits,
                                                                       r.spre, r.swords);
         }
