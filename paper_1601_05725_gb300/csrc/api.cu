@@ -68,6 +68,9 @@ struct basker_s {
     // shared memory per ND level (0: not on this level), columns it hands on
     bk_tdesc_dev td{};
     std::vector<size_t> td_smem;
+    std::vector<int32_t> td_first;   // staged: a level's first column in td_cols, the separators' columns
+    int32_t *td_cols = nullptr;
+    int32_t td_ncols = 0;
     int32_t *td_over = nullptr;
     // the arena as the symbolic pass left it (natural pivots, symbolic pattern and
     // schedule): a factorization first tries the stored-pattern path from it
@@ -427,24 +430,22 @@ int setup_teams(basker_t h)
 int setup_tdesc(basker_t h)
 {
     const bk_plan &pl = h->pl;
-    h->td_smem.assign(pl.level_tasks.size(), 0);
-    if (!h->team_path || pl.level_tasks.size() < 2 || pl.counts_only) return BASKER_OK;
-    // levels with a column of 2,000 steps or more under the natural pivots (supply
+    const size_t nl = pl.level_tasks.size();
+    h->td_smem.assign(nl, 0);
+    h->td_first.assign(nl + 1, 0);
+    if (!h->team_path || nl < 2 || pl.counts_only || h->stored_first) return BASKER_OK;
+    // unstaged: levels with a column of 2,000 steps or more under the natural pivots (supply
     // rails); fewer steps lie in one or two nodes, and one warp takes them as fast
-    std::vector<char> on(pl.level_tasks.size(), 0);
-    int64_t most = 0;
-    for (size_t l = 1; l < pl.level_tasks.size(); l++) {
+    std::vector<char> on(nl, 0);
+    int64_t most = 0, upper = 0;       // columns of a level with such a column; steps above level 1
+    for (size_t l = 1; l < nl; l++) {
         for (int32_t t : pl.level_tasks[l])
-            for (int32_t c = pl.tasks[(size_t)t].lo; c < pl.tasks[(size_t)t].hi; c++)
+            for (int32_t c = pl.tasks[(size_t)t].lo; c < pl.tasks[(size_t)t].hi; c++) {
                 if (pl.sUcnt[(size_t)c] >= 2000) on[l] = 1;
+                if (l > 1) upper = std::max<int64_t>(upper, pl.sUcnt[(size_t)c]);
+            }
         if (on[l]) most = std::max<int64_t>(most, h->lv_ncols[l]);
     }
-    if (most == 0 || h->stored_first) return BASKER_OK;
-    const int64_t rows = pl.block_ptr[(size_t)pl.nd_block + 1] - pl.block_ptr[(size_t)pl.nd_block];
-    // netlists log some thousand entries a column, a supply rail tied to a fifth of
-    // the rows two to three a row; at most 128 MB in all
-    h->td.cap = (int32_t)(std::min<int64_t>(std::max<int64_t>(4 * rows, 16384), 262144) + 63) & ~63;
-    h->td.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>({most, 304, ((int64_t)128 << 20) / ((int64_t)h->td.cap * 20)}));
     for (size_t t = 0; t < pl.tasks.size(); t++) {
         const bk_task &T = pl.tasks[t];
         if (T.sp_lo < T.lo)
@@ -452,14 +453,71 @@ int setup_tdesc(basker_t h)
     }
     h->td.nodes = (h->td.nodes + 1) & ~1;
     if (h->td.nodes > 2048) return BASKER_OK;
-    for (size_t l = 1; l < pl.level_tasks.size(); l++) {
-        size_t sm = 0;
-        for (int32_t t : pl.level_tasks[l]) {
-            const bk_task &T = pl.tasks[(size_t)t];
-            if (T.sp_lo < T.lo) sm = std::max(sm, bk_tdesc_smem(h->td, T.lo - T.sp_lo, (int64_t)T.lo - T.sp_lo + T.lspace));
+    std::vector<size_t> sm(nl, 0);
+    auto sizes = [&]() {
+        size_t worst = 0;
+        for (size_t l = 1; l < nl; l++) {
+            sm[l] = 0;
+            for (int32_t t : pl.level_tasks[l]) {
+                const bk_task &T = pl.tasks[(size_t)t];
+                if (T.sp_lo < T.lo)
+                    sm[l] = std::max(sm[l], bk_tdesc_smem(h->td, T.lo - T.sp_lo, (int64_t)T.lo - T.sp_lo + T.lspace));
+            }
+            worst = std::max(worst, sm[l]);
         }
-        h->td_smem[l] = on[l] && sm <= BK_TDESC_SMEM ? sm : 0;
+        return worst;
+    };
+    const int64_t rows = pl.block_ptr[(size_t)pl.nd_block + 1] - pl.block_ptr[(size_t)pl.nd_block];
+    // Staged where there are two levels of separators or more, with 128 steps or more in a
+    // column above the first (fewer: kernels_tdesc.cu has both sides' times): the leaves'
+    // part of every separator column in one launch, the rest of a column when the
+    // separators below it are factored.  A column's log has room for 16 entries a step (a
+    // netlist's column has some thousand), a supply rail's for 4 a row (it has two to
+    // three); 1 GB in all.
+    if (nl >= 3 && upper >= 128) {
+        std::vector<int32_t> all;
+        std::vector<int64_t> loff{0}, xoff{0};
+        for (size_t l = 1; l < nl; l++) {
+            h->td_first[l] = (int32_t)all.size();
+            for (int32_t t : pl.level_tasks[l]) {
+                const bk_task &T = pl.tasks[(size_t)t];
+                if (T.sp_lo >= T.lo) continue;
+                for (int32_t c = T.lo; c < T.hi; c++) {
+                    const int64_t u = pl.sUcnt[(size_t)c];
+                    const int64_t cap =
+                        (std::min<int64_t>(std::max<int64_t>(u < 2000 ? 16 * u : 4 * rows, 16384), 262144) + 63) & ~63;
+                    h->td.cap = std::max(h->td.cap, (int32_t)cap);
+                    all.push_back(c);
+                    loff.push_back(loff.back() + cap);
+                    xoff.push_back(xoff.back() + (((int64_t)T.space + 63) & ~(int64_t)31));
+                }
+            }
+        }
+        const size_t worst = sizes();
+        const int64_t words = (int64_t)(worst / 4) + 8;
+        if (!all.empty() && worst <= BK_TDESC_SMEM &&
+            loff.back() * 20 + xoff.back() * 8 + words * 4 * (int64_t)all.size() <= ((int64_t)1 << 30)) {
+            h->td_ncols = (int32_t)all.size();
+            h->td.words = (int32_t)words;
+            for (size_t l = 1; l < nl; l++) h->td_smem[l] = worst;
+            TRY(upload(h, &h->td_cols, all));
+            TRY(upload(h, (int64_t **)&h->td.loff, loff));
+            TRY(upload(h, (int64_t **)&h->td.xoff, xoff));
+            TRY(dalloc(h, &h->td.x, (size_t)xoff.back(), true));
+            TRY(dalloc(h, &h->td.state, (size_t)words * all.size(), true));
+            TRY(dalloc(h, &h->td.slot, (size_t)loff.back()));
+            TRY(dalloc(h, &h->td.l, (size_t)loff.back()));
+            TRY(dalloc(h, &h->td.m, (size_t)loff.back()));
+            TRY(dalloc(h, &h->td_over, (size_t)pl.n));
+            return BASKER_OK;
+        }
     }
+    if (most == 0) return BASKER_OK;
+    // a log a block, at most 128 MB in all
+    h->td.cap = (int32_t)(std::min<int64_t>(std::max<int64_t>(4 * rows, 16384), 262144) + 63) & ~63;
+    h->td.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>({most, 304, ((int64_t)128 << 20) / ((int64_t)h->td.cap * 20)}));
+    sizes();
+    for (size_t l = 1; l < nl; l++) h->td_smem[l] = on[l] && sm[l] <= BK_TDESC_SMEM ? sm[l] : 0;
     TRY(dalloc(h, &h->td.slot, (size_t)h->td.cap * (size_t)h->td.blocks));
     TRY(dalloc(h, &h->td.l, (size_t)h->td.cap * (size_t)h->td.blocks));
     TRY(dalloc(h, &h->td.m, (size_t)h->td.cap * (size_t)h->td.blocks));
@@ -841,7 +899,10 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
                 h->launches++;
             }
             if (h->td_smem[l]) {
-                bk_launch_tdesc(dl, h->td, list, ncols, cnt + 11, nlist, h->td_over, cnt + 12, h->td_smem[l], s);
+                // staged: the leaves' part of all levels' columns first, with level 1's whole
+                const int stage = !h->td.loff ? 0 : l == 1 ? 1 : 2;
+                bk_launch_tdesc(dl, h->td, stage == 1 ? h->td_cols : list, stage == 1 ? h->td_ncols : ncols, cnt + 11, nlist,
+                                h->td_over, cnt + 12, h->td_smem[l], stage, stage == 2 ? h->td_first[l] : 0, s);
                 CU(cudaGetLastError());
                 list = h->td_over;
                 nlist = cnt + 12;

@@ -227,14 +227,24 @@ struct bk_tdesc_dev {
     double *l = nullptr, *m = nullptr;
     int32_t cap = 0, blocks = 0;
     int32_t nodes = 0;               // most descendant nodes of a separator
+    // staged (loff not null): a log (cap: the longest), a vector and a saved state a column,
+    // columns by their place in the levels' lists one after the other
+    const int64_t *loff = nullptr, *xoff = nullptr;
+    double *x = nullptr;
+    uint32_t *state = nullptr;
+    int32_t words = 0;               // of a saved state
     // per L entry: where the L column of its row's step lies (start << 20 | length);
     // an array the factors by rows use later
     unsigned long long *link = nullptr;
 };
 size_t bk_tdesc_smem(const bk_tdesc_dev &lg, int64_t ndesc, int64_t space);
-// columns whose log does not fit are listed in over[0 .. *nover)
+// columns whose log does not fit are listed in over[0 .. *nover).  stage 0: cols[0 ..
+// ncols) whole; 1: cols is every separator column, their leaves' part (whole where the
+// separator has only leaves below); 2: the rest of cols[0 .. ncols), the columns from
+// `first` on of stage 1's list
 void bk_launch_tdesc(const bk_dev &d, const bk_tdesc_dev &lg, const int32_t *cols, int32_t ncols, int32_t *counter,
-                     const int32_t *ncols_dev, int32_t *over, int32_t *nover, size_t smem, void *stream);
+                     const int32_t *ncols_dev, int32_t *over, int32_t *nover, size_t smem, int stage, int first,
+                     void *stream);
 // the rows of the L columns of the ND nodes of a level as steps, for it (d.Ls)
 void bk_launch_lsteps(const bk_dev &d, const bk_tdesc_dev &lg, int32_t c0, int32_t c1, int32_t level, void *stream);
 // kernels_team.cu: Algorithm 1 on tasks without descendants, a block of W warps per

@@ -15,13 +15,23 @@
 //
 // A column whose log outgrows its room is listed for bk_gp_desc_kernel.
 //
+// In stages, where a separator has separators below it: its columns' steps in the leaves
+// need the leaves alone.  So the first launch takes every separator column of the block
+// through its leaves (level 1's columns whole) and keeps its vector, bitmaps and logs;
+// each later level's launch goes on from there when the separators below are factored.
+// One wave of leaf steps then takes the place of one a level, nearly all of a netlist
+// column's steps being in one leaf.  (A problem whose regions would take more than 1 GB,
+// or with one level of separators, takes the columns of a level whole, if at all.)
+//
 // What bounds it: a step's chain of dependent instructions and reads (about 2,500
 // cycles; 3,000 in one warp alone), so the steps of the node that has most, and the
-// walk over the logs.  A supply rail's column has 22,600 steps: the root separator
-// of the 100,003-row circuit with rails 9.5 to 12 ms, was 34.  A column of some
-// hundred steps has nearly all of them in one leaf and gains nothing: the levels
-// without a column of 2,000 symbolic steps keep bk_gp_desc_kernel (0.75 to 0.9 ms
-// either way).
+// walk over the logs.  Measured, the descendant phase of a factorization: 150,001-row
+// netlist, 32 leaves, 7.6 ms one warp a column and level by level, 3.4 in stages (2.0 for
+// the leaves); 20,011 rows, 8 leaves, 2.2 and 1.15; 100,003-row circuit with supply
+// rails of up to 22,600 steps 37 (one warp), 14.6 (columns of a level whole, rails only),
+// 12.8 in stages.  With columns of fewer than 128 symbolic steps above level 1 the stages'
+// own work shows: 2,000-row circuit, 4 leaves, 0.10 ms a level in one warp, 0.16 here.
+// 1,024 threads a block spill registers and put one block on an SM: 3.4 ms for the leaves.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,7 +45,7 @@ using namespace bk;
 
 namespace {
 
-constexpr int TD_NT = 1024;
+constexpr int TD_NT = 512;
 constexpr int TD_W = TD_NT / 32;
 constexpr int TD_CK = 64;              // entries of a log chunk
 
@@ -44,7 +54,8 @@ constexpr int TD_CK = 64;              // entries of a log chunk
 template <typename V>
 __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t *__restrict__ cols, int32_t ncols,
                                                          int32_t *counter, const int32_t *__restrict__ ncols_dev,
-                                                         int32_t *over, int32_t *nover, bk_tdesc_dev lg)
+                                                         int32_t *over, int32_t *nover, bk_tdesc_dev lg, int stage,
+                                                         int first)
 {
     if (ncols_dev) ncols = *ncols_dev;
     extern __shared__ __align__(16) uint32_t td_sm[];
@@ -57,17 +68,12 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
     V *const Ahat = vals<V>(d.ahat);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    const int nchunks = lg.cap / TD_CK;
-    int32_t *const log_s = lg.slot + (int64_t)blockIdx.x * lg.cap;
-    V *const log_l = vals<V>(lg.l) + (int64_t)blockIdx.x * lg.cap;
-    V *const log_m = vals<V>(lg.m) + (int64_t)blockIdx.x * lg.cap;
-    V *const x = reinterpret_cast<V *>(d.wsd + (int64_t)blockIdx.x * d.wsd_slice);
     // per descendant node two logs: to descendant rows (2 D), and to the separator's
     // and its ancestors' (2 D + 1): first chunk and entries
     int32_t *const nfirst = reinterpret_cast<int32_t *>(td_sm);
     int32_t *const ncnt = nfirst + 2 * lg.nodes;
     uint16_t *const next = reinterpret_cast<uint16_t *>(ncnt + 2 * lg.nodes);
-    volatile uint32_t *const sb = td_sm + 4 * lg.nodes + ((nchunks + 1) >> 1);
+    volatile uint32_t *const sb = td_sm + 4 * lg.nodes + ((lg.cap / TD_CK + 1) >> 1);
     for (;;) {
         __syncthreads();
         if (tid == 0) {
@@ -76,11 +82,21 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
         }
         __syncthreads();
         if (s_col >= ncols) return;
-        const int c = cols[s_col];
+        const int ord = stage == 1 ? ncols - 1 - s_col : first + s_col;
+        const int c = cols[stage == 1 ? ord : s_col];
+        const int64_t lg0 = stage ? lg.loff[ord] : (int64_t)blockIdx.x * lg.cap;
+        const int nchunks = (stage ? (int)(lg.loff[ord + 1] - lg0) : lg.cap) / TD_CK;
+        int32_t *const log_s = lg.slot + lg0;
+        V *const log_l = vals<V>(lg.l) + lg0;
+        V *const log_m = vals<V>(lg.m) + lg0;
+        V *const x = stage ? vals<V>(lg.x) + lg.xoff[ord] : reinterpret_cast<V *>(d.wsd + (int64_t)blockIdx.x * d.wsd_slice);
+        uint32_t *const keep = lg.state + (int64_t)ord * lg.words;
         const int task = d.col_task[c];
         if (wid == 0) load_task(T, d.tasks + task, lane);
         __syncthreads();
-        if (__syncthreads_or(tid == 0 && should_stop(d, task, c))) continue;
+        const bool quit = __syncthreads_or(tid == 0 && should_stop(d, task, c));
+        if (quit && stage < 2) continue;
+        const bool part = stage == 1 && T.level > 1;      // the leaves only, for stage 2
         const int base = T.sp_lo;
         const int ndesc = T.lo - base;
         const int lsp = T.lspace;
@@ -89,10 +105,20 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
         volatile uint32_t *const pr = ap + nsw;
         const int t0 = d.col_task[base];               // the descendants: tasks [t0, task)
         const int nn = task - t0;
-        for (int i = tid; i < 2 * nsw + npw; i += TD_NT) sb[i] = 0u;
-        for (int i = tid; i < 2 * nn; i += TD_NT) {
-            nfirst[i] = -1;
-            ncnt[i] = 0;
+        const int words = (int)(sb - td_sm) + 2 * nsw + npw;
+        if (stage < 2) {
+            for (int i = tid; i < 2 * nsw + npw; i += TD_NT) sb[i] = 0u;
+            for (int i = tid; i < 2 * nn; i += TD_NT) {
+                nfirst[i] = -1;
+                ncnt[i] = 0;
+            }
+        } else {
+            for (int i = tid; i < words; i += TD_NT) td_sm[i] = keep[4 + i];
+            if (tid == 0) {
+                s_chunks = (int)keep[0];
+                s_bad = (int)keep[1];
+                s_over = (int)keep[2];
+            }
         }
         __syncthreads();
         auto bit_set = [](volatile uint32_t *w, int i) {
@@ -103,9 +129,12 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
             const int r = d.Bi[e];
             const int s = slot_of(T, base, r);
             if (s < 0) { report_internal(d.status, c, 61); continue; }
-            x[s] = Bx[e];
-            bit_set(pr, s);
-            if (s < ndesc) {
+            if (stage < 2) {
+                x[s] = Bx[e];
+                bit_set(pr, s);
+            }
+            // (the rows of separators below have their pivots by stage 2)
+            if (s < ndesc && !quit && (stage == 0 || !(d.tasks[d.col_task[r]].level == 0 ? stage == 2 : part))) {
                 const int p = d.pinv[r] - base;
                 if ((unsigned)p < (unsigned)ndesc) bit_set(sb, p);
                 else report_internal(d.status, c, 62);
@@ -156,7 +185,7 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
             }
         };
 
-        for (int h = 0; h < T.level; h++) {
+        for (int h = stage == 2 ? 1 : 0; h < (quit ? 0 : part ? 1 : T.level); h++) {
             for (int D = wid; D < nn; D += TD_W) {
                 const bk_task *const N = d.tasks + t0 + D;
                 if (__any_sync(BK_FULL, N->level != h || s_over)) continue;
@@ -345,13 +374,24 @@ __global__ void __launch_bounds__(TD_NT) bk_tdesc_kernel(bk_dev d, const int32_t
             }
             __syncthreads();
         }
-        if (!s_over) {
+        if (part) {
+            // the rest when the separators below are factored
+            for (int i = tid; i < words; i += TD_NT) keep[4 + i] = td_sm[i];
+            if (tid == 0) {
+                keep[0] = (uint32_t)s_chunks;
+                keep[1] = (uint32_t)s_bad;
+                keep[2] = (uint32_t)s_over;
+            }
+            continue;
+        }
+        if (!s_over && !quit) {
             // the separator's and its ancestors' rows: a warp takes every TD_W-th slot
             for (int D = 0; D < nn; D++)
                 take_log(2 * D + 1, [&](int s) { return (s & (TD_W - 1)) == wid; }, false);
         }
         __syncthreads();
-        if (s_over) {
+        if (quit) {
+        } else if (s_over) {
             if (tid == 0) over[atomicAdd(nover, 1)] = c;
         } else {
             // U(desc, c): the applied steps in ascending order, a run of words a thread
@@ -452,7 +492,8 @@ void bk_launch_lsteps(const bk_dev &d, const bk_tdesc_dev &lg, int32_t c0, int32
 }
 
 void bk_launch_tdesc(const bk_dev &d, const bk_tdesc_dev &lg, const int32_t *cols, int32_t ncols, int32_t *counter,
-                     const int32_t *ncols_dev, int32_t *over, int32_t *nover, size_t smem, void *stream)
+                     const int32_t *ncols_dev, int32_t *over, int32_t *nover, size_t smem, int stage, int first,
+                     void *stream)
 {
     if (ncols <= 0) return;
     static std::once_flag once;
@@ -460,8 +501,11 @@ void bk_launch_tdesc(const bk_dev &d, const bk_tdesc_dev &lg, const int32_t *col
         cudaFuncSetAttribute(bk_tdesc_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, BK_TDESC_SMEM);
         cudaFuncSetAttribute(bk_tdesc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, BK_TDESC_SMEM);
     });
-    const int grid = std::min(std::min(ncols, lg.blocks), d.wsd_warps);
+    // staged: a region a column; else a region a block
+    const int grid = stage ? std::min(ncols, 608) : std::min(std::min(ncols, lg.blocks), d.wsd_warps);
     cudaStream_t s = (cudaStream_t)stream;
-    if (d.prec) bk_tdesc_kernel<float><<<grid, TD_NT, smem, s>>>(d, cols, ncols, counter, ncols_dev, over, nover, lg);
-    else bk_tdesc_kernel<double><<<grid, TD_NT, smem, s>>>(d, cols, ncols, counter, ncols_dev, over, nover, lg);
+    if (d.prec)
+        bk_tdesc_kernel<float><<<grid, TD_NT, smem, s>>>(d, cols, ncols, counter, ncols_dev, over, nover, lg, stage, first);
+    else
+        bk_tdesc_kernel<double><<<grid, TD_NT, smem, s>>>(d, cols, ncols, counter, ncols_dev, over, nover, lg, stage, first);
 }
