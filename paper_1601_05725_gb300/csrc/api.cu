@@ -36,6 +36,7 @@ struct basker_s {
     std::vector<bk_team_group> team;
     bool team_path = false;      // every level-0 task has a team, every separator a dense elimination
     bool stored_first = false;   // the stored-pattern pass before the teams (dense enough columns)
+    bool settled = false;        // the last refactorization moved no pivot
     bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones)
     bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once from then on
     // separators whose in-node phase runs as one dense elimination, by kernel and cluster size
@@ -866,13 +867,15 @@ int launch_leaves(basker_t h, cudaStream_t s, int pref_mode, bool repair)
 
 // The separators above level 0, level by level (Algorithm 4's dependency tree).
 // stored: the descendant phase starts from the stored patterns (verified on the
-// device), else every column takes the reach.
-int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
+// device), else every column takes the reach.  same: the level-0 tasks moved no pivot, so
+// that the stored patterns will do for thin columns and rails as well.
+int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bool same)
 {
     const int32_t nd0 = h->pl.nd_block >= 0 ? h->pl.block_ptr[(size_t)h->pl.nd_block] : 0;
     const int32_t nd1 = h->pl.nd_block >= 0 ? h->pl.block_ptr[(size_t)h->pl.nd_block + 1] : 0;
     for (size_t l = 1; l < h->lv_tasks.size(); l++) {
-        if (h->td.slot) {
+        const size_t td_smem = same ? 0 : h->td_smem[l];
+        if (h->td.slot && !same) {
             tbeg(h, KT_DESC, s, 1);
             bk_launch_lsteps(h->d, h->td, nd0, nd1, (int32_t)l - 1, s);
             CU(cudaGetLastError());
@@ -888,9 +891,9 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
             const int32_t ncols = h->lv_ncols[l];
             // (a rail's column is 22,000 steps one after the other on its stored pattern:
             // the reach with its nodes in parallel takes less)
-            const bk_desc_par par = stored && l < h->df_par.size() && !h->td_smem[l] ? h->df_par[l] : bk_desc_par{};
+            const bk_desc_par par = stored && l < h->df_par.size() && !td_smem ? h->df_par[l] : bk_desc_par{};
             CU(cudaMemsetAsync(cnt, 0, 16 * sizeof(int32_t), s));
-            tbeg(h, KT_DESC, s, (par.smem > 0) + (h->td_smem[l] > 0) + 1);
+            tbeg(h, KT_DESC, s, (par.smem > 0) + (td_smem > 0) + 1);
             if (par.smem) {
                 bk_launch_desc_fast(dl, list, ncols, cnt + 5, h->df_redo, cnt + 7, par, s);
                 CU(cudaGetLastError());
@@ -898,11 +901,11 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored)
                 nlist = cnt + 7;
                 h->launches++;
             }
-            if (h->td_smem[l]) {
+            if (td_smem) {
                 // staged: the leaves' part of all levels' columns first, with level 1's whole
                 const int stage = !h->td.loff ? 0 : l == 1 ? 1 : 2;
                 bk_launch_tdesc(dl, h->td, stage == 1 ? h->td_cols : list, stage == 1 ? h->td_ncols : ncols, cnt + 11, nlist,
-                                h->td_over, cnt + 12, h->td_smem[l], stage, stage == 2 ? h->td_first[l] : 0, s);
+                                h->td_over, cnt + 12, td_smem, stage, stage == 2 ? h->td_first[l] : 0, s);
                 CU(cudaGetLastError());
                 list = h->td_over;
                 nlist = cnt + 12;
@@ -1372,13 +1375,25 @@ int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool 
         if (st != BASKER_OK) return st;
         stored = h->h_status->repaired <= many;
     }
-    TRY(launch_separators(h, s, pref_mode, stored));
+    bool same = false;
+    if (first && !h->stored_first && h->lv_tasks.size() > 1) {
+        const int st = read_status(h, s);
+        if (st != BASKER_OK) {
+            h->settled = h->patterns_hold = h->leaf_levels = false;
+            h->order_stale = true;
+            return st;
+        }
+        same = h->h_status->static_fail == 0;
+    }
+    TRY(launch_separators(h, s, pref_mode, stored, same));
     const int st = read_status(h, s);
     h->patterns_hold = h->leaf_levels = st == BASKER_OK;
     if (st == BASKER_OK && first && h->h_status->static_fail == 0) h->schedule_valid = true;   // no pattern moved
     else h->order_stale = true;
+    h->settled = false;
     if (st == BASKER_OK) {
         note_repair(h);
+        h->settled = pref_mode && (first ? h->h_status->static_fail : h->h_status->repaired) == 0;
         if (first && h->h_status->static_fail > many) h->many_rejects = true;
     }
     return st;
@@ -1409,7 +1424,12 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         int st = BASKER_OK;
         if (teams) {
             bool stored = true;
-            const bool first = h->stored_first && h->patterns_hold && !h->many_rejects && h->opt.refactor_switch == 0;
+            // the stored-pattern pass first where columns are dense, and for any pattern
+            // once a refactorization has moved no pivot (a sequence that repeats, or moves
+            // little: a pass of three 25,162-row circuits with rails 21.9 ms by teams and
+            // stages, 13.2 so; two 137,468-row netlists 24.8 and 21.4)
+            const bool first = (h->stored_first || h->settled) && h->patterns_hold && !h->many_rejects &&
+                               h->opt.refactor_switch == 0;
             st = factor_by_teams(h, s, 1, first, stored);
             if (st == BASKER_ERR_TIMEOUT) {
                 // the pivots of before, for the next call

@@ -58,7 +58,7 @@ struct bk_status {
     int32_t offdiag;                 // number of columns pivoting off the natural row
     int32_t internal_site;           // first internal-consistency check that fired (0 = none)
     int32_t internal_col;            // and its column
-    int32_t repaired;                // columns recomputed by the repair kernel
+    int32_t repaired;                // columns a repair recomputed, or teams gave another pivot
     int32_t pad;
 };
 

@@ -73,3 +73,28 @@ def test_failure_between_the_stages(node):
     assert o.factor(prob.values) == "OK"
     h.factor(_dev(prob.values))
     _same(h, o.factors())
+
+
+@pytest.mark.parametrize("make", [
+    lambda: I.netlist_problem(94, n_small=60, m_netlist=20000, depth=2),
+    lambda: I.config4(95, n=9000, n_rails=4, rail_deg=(2500, 4000)),
+    lambda: I.block_diagonal_problem(96, nblocks=60, size_range=(1, 500)),
+])
+def test_sequence_that_settles_and_moves_again(make):
+    """Values repeated until no pivot moves (the stored patterns serve), then new ones."""
+    prob = make()
+    o = oracle.OracleLU(prob)
+    assert o.factor() == "OK"
+    f = o.factors()
+    h = basker.Handle.from_problem(prob)
+    h.factor(_dev(prob.values))
+    static = 0
+    for k in (1, 1, 1, 2, 2, 2, 1):
+        v = I.refactor_values(prob, k, sigma=0.3)
+        assert o.factor(v, pref=f.prow) == "OK"
+        f = o.factors()
+        h.info()
+        h.refactor(_dev(v))
+        static += h.info()["kernel_calls"]["static_refactor"]
+        _same(h, f)
+    assert static > 0, "no refactorization on the stored patterns"
