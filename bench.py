@@ -362,19 +362,17 @@ def _measure(h, dvals, drhs, K, W, dev, flush, dist, world):
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one
 # ncu capture of the kernel as it stands, by kernel kind and value width.  A kind
 # without a capture of its current code reports null.
-TRAFFIC = {("powergrid_316x316", "solve", 8): 102.8e6, ("powergrid_316x316", "refactor_rounds", 8): 19.2e6,
-           ("powergrid_316x316", "dense_node", 8): 2.3e6}
+TRAFFIC = {}
 # sm__pipe_fp64_cycles_active (pct of peak) from the same captures
-FP64_PIPE = {("powergrid_316x316", "solve", 8): 16.5, ("powergrid_316x316", "refactor_rounds", 8): 1.4,
-             ("powergrid_316x316", "dense_node", 8): 24.1}
+FP64_PIPE = {}
 
 
 def _roofline(prob, info1, K, nnz_lu, vbytes, hbm):
     """HBM roofline of the kernel kind with the most device time per step.
 
     Algorithmic bytes (values vbytes wide, indices 4 B): a refactorization moves
-    (vbytes + 4)(|A| + |L+U|); a refactorization round moves that share of it
-    which its columns hold (columns processed / n, per round launch); a solve
+    (vbytes + 4)(|A| + |L+U|); a repair (or a round) moves that share of it which
+    the columns it computes hold (columns / n, per launch); a solve
     (vbytes + 4)|L+U| + 24 n per right-hand side."""
     kms = {k: v for k, v in info1["kernel_ms"].items() if v > 0}
     calls = info1["kernel_calls"]
@@ -455,8 +453,8 @@ def _latency_floor(prob, h, kinds_ms, info1, K, probe):
     (probe: flag handoff H, dependent FP64 fma F, FP64 division D): a solve row
     H + F forward, H + F + D backward; a factorization column H + F + D (its last
     step's update, its pivot, the division of its L column); a column level H; a
-    dense elimination step F + D (no handoff: one cluster); the rounds repeat the
-    leaves' column chain once per launch."""
+    dense elimination step F + D (no handoff: one cluster); a repair (or a round)
+    walks the leaves' column chain once a launch, as does Algorithm 1 by teams."""
     _, L, U = h.export()
     dep = _chain_depths(prob, L, U)
     H, F, D = probe["flag_handoff_ns"], probe["dfma_ns"], probe["ddiv_ns"]
@@ -465,6 +463,7 @@ def _latency_floor(prob, h, kinds_ms, info1, K, probe):
                        dep["forward_rows"] + dep["columns"]),
              "static_refactor": (dep["columns"] * (H + F + D), dep["columns"]),
              "dag_levels": (dep["columns"] * H, dep["columns"]),
+             "gp_in_node": (dep["leaf_columns"] * (H + F + D), dep["leaf_columns"]),
              "refactor_rounds": (rounds_per_step * dep["leaf_columns"] * (H + F + D),
                                  rounds_per_step * dep["leaf_columns"]),
              "dense_node": (dep["separator_steps"] * (F + D), dep["separator_steps"])}

@@ -76,21 +76,29 @@ typedef struct {
     double ir_tol;                /* precision 1, 2: backward error to reach; default 1e-13 */
     double growth_limit;          /* precision 1: max over BTF blocks of max|U_d| / max|B_d|
                                      above which the FP32 factors are not used; default 1e4 */
-    int refactor_switch;          /* the pivots a refactorization's stored-pattern pass
-                                     rejected are resolved, 0 (default): by rounds of
-                                     column recomputation until they have taken as long
-                                     as the handle's last complete factorization, the rest
-                                     then one complete Algorithm 1 pass with the previous
-                                     pivots preferred (that pass at once when more than
-                                     max(16, n/200) pivots were rejected); 1: rounds
-                                     only; 2: the complete
-                                     pass at once; 3: when every ND separator fits the
-                                     dense elimination, the repair pass (one block of
+    int refactor_switch;          /* 0 (default): where every ND separator fits the dense
+                                     elimination, the ND leaves and BTF blocks are factored
+                                     by teams (a block of warps per task, columns in flight
+                                     together); patterns with dense columns (32 symbolic L
+                                     and U entries a column or more), and any pattern once
+                                     a refactorization has moved no pivot, run the
+                                     stored-pattern pass first and teams repair from each
+                                     task's first rejected pivot on, until a pass rejects
+                                     too many.
+                                     Elsewhere a stored-pattern pass and rounds of column
+                                     recomputation until they have taken as long as the
+                                     handle's last complete factorization, the rest then
+                                     one complete Algorithm 1 pass with the previous pivots
+                                     preferred (that pass at once when more than
+                                     max(16, n/200) pivots were rejected); 1: stored-pattern
+                                     pass and rounds only; 2: teams without a stored-pattern
+                                     pass, or elsewhere the complete pass at once; 3: when
+                                     every ND separator fits the dense elimination, the
+                                     stored-pattern pass and the repair pass (one block of
                                      threads per ND leaf or BTF block walks its columns
-                                     from the first rejection on, in column order, on the
-                                     device, with no host round trip), else as 0.  The
-                                     factors are the same in every mode (other values:
-                                     INVALID_ARG). */
+                                     from the first rejection on, in column order), else as
+                                     0.  The factors are the same in every mode (other
+                                     values: INVALID_ARG). */
     int graphs;                   /* nonzero (default): the launches that follow every
                                      factorization are replayed from a CUDA graph captured
                                      once per L/U arena; 0: launched one by one */
@@ -121,7 +129,8 @@ typedef struct {
     int64_t nnz_l_sym, nnz_u_sym; /* symbolic counts under the preferred (diagonal) pivots */
     double flops;                 /* sum_j l_j (2 u_j + 1) of the current factors */
     int32_t failed_column;        /* column named by SINGULAR / NAN, else -1 */
-    int32_t last_repivot_columns; /* columns recomputed by the reach in the last refactor */
+    int32_t last_repivot_columns; /* last refactor: columns that teams or repair gave another
+                                     pivot than preferred, or that rounds recomputed */
     int32_t off_diagonal_pivots;  /* columns whose pivot is not the natural row */
     int32_t capacity_regrows;     /* times the L/U arena was regrown */
     int64_t device_bytes;         /* device memory held by the handle */
@@ -131,16 +140,18 @@ typedef struct {
     double kernel_ms[10];         /* with options.timing: device time per kernel kind since
                                      the last basker_info call: [0] value gather,
                                      [1] stored-pattern refactor, [2] DAG levels,
-                                     [3] in-node Algorithm 1, [4] separator descendant
+                                     [3] in-node Algorithm 1 (by
+                                     teams, or a warp a task), [4] separator descendant
                                      phase, [5] solve, [6] separators' in-node phase as
                                      dense eliminations,
-                                     [7] refactorization rounds after the stored-pattern
-                                     pass, [8] factors transposed into rows for the
+                                     [7] what follows a stored-pattern pass on the leaves
+                                     and blocks (repair by teams, rounds), [8] factors transposed into rows for the
                                      solve, [9] FP64 refinement (precision 1) */
     int32_t internal_site;        /* nonzero: code of the internal consistency check that
                                      failed (reported as INVALID_ARG), for diagnosis */
     int32_t internal_col;         /* column of that check */
-    int32_t last_rounds;          /* redo rounds of the last refactor (0: no pivot rejected) */
+    int32_t last_rounds;          /* redo rounds of the last refactor, 1 for a repair (0: no
+                                     pivot rejected) */
     int32_t ir_iterations;        /* precision 1: refinement steps of the last solve */
     int32_t ir_fallbacks;         /* precision 1: factorizations redone in FP64 so far */
     int32_t precision_used;       /* arithmetic of the factors the last solve used: 0 FP64, 1 FP32 */
@@ -153,10 +164,12 @@ typedef struct {
     int32_t cuda_error;           /* after a CUDA status: the runtime's error code of the last
                                      failing call made by this thread, and */
     int32_t cuda_line;            /* the library source line of that call (diagnosis) */
-    int64_t rounds_columns;       /* columns processed by refactorization rounds since the
-                                     last basker_info call */
+    int64_t rounds_columns;       /* columns processed by rounds, recomputed by a repair or
+                                     given another pivot by teams, since the last
+                                     basker_info call */
     int32_t full_refactors;       /* refactorizations finished by a complete Algorithm 1
-                                     pass instead of rounds (options.refactor_switch) */
+                                     pass instead of rounds (options.refactor_switch), or by
+                                     teams under refactor_switch 2 with a pivot moved */
     int32_t graph_launches;       /* CUDA graph replays so far (options.graphs) */
     int32_t static_factors;       /* basker_factor calls served by the stored-pattern path
                                      (natural pivots preferred) instead of a complete pass */
@@ -208,11 +221,9 @@ int basker_symbolic(int32_t n, const int32_t *colptr, const int32_t *rowind,
 int basker_factor(basker_t h, const double *values_dev, void *stream);
 
 /* Refactorization of a new matrix with the same pattern (Sec. V): each column
- * prefers the pivot row of the previous factorization; columns that keep it are
- * computed on the stored pattern (column-level dataflow), and a node whose
- * column rejects its preferred pivot is recomputed from that column on with the
- * reach of Algorithm 1, together with its ancestors.  The result equals a fresh
- * factorization with those preferences.  Errors as basker_factor, and
+ * prefers the pivot row of the previous factorization (options.refactor_switch:
+ * which columns are computed on the stored pattern and which by the reach of
+ * Algorithm 1).  The result equals a fresh factorization with those preferences.  Errors as basker_factor, and
  * NOT_FACTORED. */
 int basker_refactor(basker_t h, const double *values_dev, void *stream);
 
@@ -269,7 +280,7 @@ int basker_probe_latency(double *ns_out);
  *   The solve's two work vectors (the forward results and the solution by
  *   pivot step, n * nrhs doubles each) live in one array of
  *   BASKER_NOALLOC_SCRATCH_DOUBLES doubles compiled into the library; its other
- *   buffers (per-row flags, the factors by rows) are the handle's, made when it
+ *   buffers (the separators' partial sums, the factors by rows) are the handle's, made when it
  *   was factored.  So the call performs no cudaMalloc, cudaFree or other
  *   allocation.  It needs 2 * nrhs * n doubles; larger requests return
  *   BASKER_ERR_INVALID_ARG without launching anything, and so does a handle with
