@@ -42,7 +42,8 @@ struct bk_task {
     int64_t wsoff;             // offset (bytes) of x + bitmaps in the global workspace, -1 = shared
     int64_t ahoff;             // separators: first double of the task's A-hat columns (lspace each)
     int64_t aboff;             // separators: first word of their pattern bitmaps (ceil(lspace/32) each)
-    int32_t level;             // height in the ND tree (0: leaves and small BTF blocks)
+    int32_t level;             // height in the ND tree (0: leaves, BTF blocks, and separators whose
+                               // descendants are all empty)
     int32_t node;              // ND node (postorder) or -1
     int32_t block;             // BTF block
     int32_t dense;             // separators: refactorizations recompute it by the descendant

@@ -208,7 +208,8 @@ static void interval_counts(bk_plan &pl)
     SymTree st;
     sym_tree(pl, st);
     auto task_of = [&](int32_t c) -> const bk_task & { return pl.tasks[(size_t)pl.col_task[(size_t)c]]; };
-    auto exact = [&](int32_t c) { return task_of(c).level == 0; };
+    auto height = [&](const bk_task &T) { return T.node < 0 ? 0 : pl.nd_height[(size_t)T.node]; };
+    auto exact = [&](int32_t c) { return height(task_of(c)) == 0; };
     // lest: per column, one range per ancestor node and one for its own node
     std::vector<int64_t> off((size_t)n + 1, 0);
     for (int32_t c = 0; c < n; c++) off[(size_t)c + 1] = off[(size_t)c] + task_of(c).nanc + 1;
@@ -255,7 +256,7 @@ static void interval_counts(bk_plan &pl)
     }
     // separators, children before parents (the tasks are in postorder)
     for (const bk_task &J : pl.tasks) {
-        if (J.level == 0 || J.node < 0) continue;
+        if (height(J) == 0) continue;
         const int32_t m = J.hi - J.lo, ns = J.nanc, w = ns + 1;     // ranges: ancestors, then own
         std::vector<int32_t> cnt((size_t)m, 0), rmin((size_t)m * w, INT32_MAX), rmax((size_t)m * w, -1);
         auto hull = [&](int32_t c, int32_t q, int32_t lo, int32_t hi) {
@@ -448,7 +449,8 @@ int bk_plan_build(int32_t n, const int32_t *colptr, const int32_t *rowind, const
                 T.space = (T.hi - T.sp_lo) + (lsp - (T.hi - T.lo));
                 T.lspace = lsp;
                 bk_task_ranges(T);
-                T.level = pl.nd_height[(size_t)t];
+                // a separator whose descendants are all empty waits for nothing: a leaf
+                T.level = T.sp_lo < T.lo ? pl.nd_height[(size_t)t] : 0;
                 T.node = t;
                 T.block = d;
                 maxlevel = std::max(maxlevel, T.level);
