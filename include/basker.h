@@ -224,7 +224,9 @@ int basker_factor(basker_t h, const double *values_dev, void *stream);
  * prefers the pivot row of the previous factorization (options.refactor_switch:
  * which columns are computed on the stored pattern and which by the reach of
  * Algorithm 1).  The result equals a fresh factorization with those preferences.  Errors as basker_factor, and
- * NOT_FACTORED. */
+ * NOT_FACTORED.  After SINGULAR, NAN, OOM or TIMEOUT the handle has no factors to solve with;
+ * after TIMEOUT it still has the pivots it started from, so that a refactorization may follow
+ * (after the others, a factorization). */
 int basker_refactor(basker_t h, const double *values_dev, void *stream);
 
 /* Solve A X = B for nrhs right-hand sides (column-major, leading dimensions ldb,

@@ -37,7 +37,8 @@ struct basker_s {
     bool team_path = false;      // every level-0 task has a team, every separator a dense elimination
     bool stored_first = false;   // the stored-pattern pass before the teams (dense enough columns)
     bool settled = false;        // the last refactorization moved no pivot
-    bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones)
+    bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones):
+                                 // a stored-pattern pass may start from them
     bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once from then on
     // separators whose in-node phase runs as one dense elimination, by kernel and cluster size
     // (bk_dense_node_group)
@@ -51,6 +52,7 @@ struct basker_s {
     int32_t *h_task_fail = nullptr;  // pinned
     int32_t epoch = 0, refno = 0;
     bool factored = false, ws_dirty = false, schedule_valid = true, order_is_symbolic = true;
+    bool pivots_kept = false;    // a refactorization's wait gave up: no factors, but the pivots it started from
     bool leaf_levels = false;    // the teams wrote the leaves' column levels (all the solve reads)
     bool order_stale = false;    // the stored claim order does not belong to the stored levels
     double gp_wall_ms = 0.0;     // wall time of the last complete Algorithm 1 pass (host clock)
@@ -934,7 +936,7 @@ int launch_full_gp(basker_t h, cudaStream_t s, int pref_mode)
 {
     const double tau = h->opt.tau;
     h->leaf_levels = false;
-    h->patterns_hold = true;       // nothing but a finished pass leads back to the teams
+    h->patterns_hold = false;
     CU(cudaMemsetAsync(h->d.pinv, 0xff, sizeof(int32_t) * (size_t)h->pl.n, s));
     for (size_t l = 0; l < h->lv_tasks.size(); l++) {
         if (l > 0 && h->lv_ncols[l] > 0) {
@@ -1313,6 +1315,28 @@ int factor_static(basker_t h, cudaStream_t s)
     return BASKER_OK;
 }
 
+// Algorithm 1 on every column with the previous pivots preferred: the
+// refactorization's definition, computed directly.
+int refactor_completely(basker_t h, cudaStream_t s)
+{
+    h->info.full_refactors++;
+    h->schedule_valid = false;
+    h->ws_dirty = true;
+    TRY(reset_status(h, s));
+    const auto t0 = std::chrono::steady_clock::now();
+    TRY(launch_full_gp(h, s, 1));
+    int st = read_status(h, s);
+    if (st == BASKER_OK)
+        h->gp_wall_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+    for (int tries = 0; st == -1 && tries < 16; tries++) {
+        TRY(regrow(h));
+        TRY(reset_status(h, s));
+        TRY(launch_full_gp(h, s, 1));
+        st = read_status(h, s);
+    }
+    return st;
+}
+
 // A refactorization's rejected pivots by rounds of the round kernel (host-driven
 // level by level; options.refactor_switch decides when the rest becomes one
 // complete pass), after the stored-pattern pass.  Returns the final status
@@ -1333,18 +1357,7 @@ int refactor_by_rounds(basker_t h, cudaStream_t s)
     st = full_now ? BK_SWITCH_TO_FULL : launch_redo(h, s);
     if (st == BASKER_OK) st = read_status(h, s);
     h->schedule_valid = false;
-    if (st == BK_SWITCH_TO_FULL) {
-        // Algorithm 1 on every column with the previous pivots preferred: the
-        // refactorization's definition, computed directly
-        h->info.full_refactors++;
-        h->ws_dirty = true;
-        TRY(reset_status(h, s));
-        const auto t0 = std::chrono::steady_clock::now();
-        TRY(launch_full_gp(h, s, 1));
-        st = read_status(h, s);
-        if (st == BASKER_OK)
-            h->gp_wall_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-    }
+    if (st == BK_SWITCH_TO_FULL) return refactor_completely(h, s);
     for (int tries = 0; st == -1 && tries < 16; tries++) {
         // the new pivots need more room: grow and run Algorithm 1 everywhere
         TRY(regrow(h));
@@ -1414,7 +1427,8 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
                            cudaMemcpyDeviceToDevice, s));
         // options.refactor_switch 0, or 2 (the complete pass at once)
         const bool teams = h->team_path && h->d.lpool_end < INT32_MAX && h->opt.refactor_switch % 2 == 0;
-        if (!teams) {
+        const bool from_patterns = !teams && h->patterns_hold;
+        if (from_patterns) {
             if (!h->schedule_valid) TRY(compute_schedule(h, s));
             TRY(static_pass(h, s));
             h->leaf_levels = false;
@@ -1431,12 +1445,6 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
             const bool first = (h->stored_first || h->settled) && h->patterns_hold && !h->many_rejects &&
                                h->opt.refactor_switch == 0;
             st = factor_by_teams(h, s, 1, first, stored);
-            if (st == BASKER_ERR_TIMEOUT) {
-                // the pivots of before, for the next call
-                CU(cudaMemcpyAsync(h->d.prow, h->d.pref, sizeof(int32_t) * (size_t)h->pl.n,
-                                   cudaMemcpyDeviceToDevice, s));
-                return st;
-            }
             for (int tries = 0; st == -1 && tries < 16; tries++) {
                 TRY(regrow(h));
                 TRY(reset_status(h, s));
@@ -1447,6 +1455,9 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
                 h->info.full_refactors++;
                 h->info.last_rounds = 0;
             }
+        } else if (!from_patterns) {
+            // a wait of the last refactorization gave up: no pattern to start from
+            st = refactor_completely(h, s);
         } else if (use_repair(h)) {
             // the stored-pattern pass, the repair pass and the separators run back to
             // back on the device; the status is read once at the end
@@ -1463,9 +1474,21 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
             }
         } else {
             st = refactor_by_rounds(h, s);
-            if (st == BASKER_ERR_TIMEOUT) return st;
         }
-        if (st != BASKER_OK) { h->factored = false; return st == -1 ? BASKER_ERR_OOM : st; }
+        if (st != BASKER_OK) {
+            h->factored = false;
+            if (st == BASKER_ERR_TIMEOUT) {
+                // what the call wrote is no factorization; the next refactorization starts
+                // from the pivots of before, and from no pattern
+                CU(cudaMemcpyAsync(h->d.prow, h->d.pref, sizeof(int32_t) * (size_t)h->pl.n,
+                                   cudaMemcpyDeviceToDevice, s));
+                h->pivots_kept = true;
+                h->settled = h->patterns_hold = h->leaf_levels = h->schedule_valid = false;
+                h->order_stale = true;
+            }
+            return st == -1 ? BASKER_ERR_OOM : st;
+        }
+        h->patterns_hold = true;
         TRY(finish_factorization(h, s));
         h->factored = true;
         return BASKER_OK;
@@ -1510,11 +1533,15 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
             h->factored = false;
             return st == -1 ? BASKER_ERR_OOM : st;
         }
+        // (the teams have written some of the leaves' levels)
+        h->order_is_symbolic = false;
+        h->order_stale = true;
     } else {
         st = factor_static(h, s);
     }
     if (st == BASKER_OK) {
         h->info.static_factors++;
+        h->patterns_hold = true;
         TRY(finish_factorization(h, s));
         h->factored = true;
         return BASKER_OK;
@@ -1542,6 +1569,7 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
     // with the natural pivots everywhere the pattern is the symbolic one, whose
     // static schedule is already on the device
     h->schedule_valid = (h->h_status->offdiag == 0 && h->order_is_symbolic);
+    h->patterns_hold = true;
     TRY(finish_factorization(h, s));
     h->factored = true;
     return BASKER_OK;
@@ -1559,6 +1587,9 @@ int ensure_solve_buffers(basker_t h, int32_t nrhs)
     return BASKER_OK;
 }
 
+// A refactorization has pivots to start from.
+bool has_pivots(basker_t h) { return h->factored || h->pivots_kept; }
+
 // ---- precision 1: FP32 factorization, FP64 refinement
 
 int ensure_twin(basker_t h)
@@ -1575,8 +1606,8 @@ int ensure_twin(basker_t h)
 int factor_twin(basker_t h, cudaStream_t s)
 {
     TRY(ensure_twin(h));
-    const int st = h->twin->factored ? basker_refactor(h->twin, h->d_vals64, s)
-                                     : basker_factor(h->twin, h->d_vals64, s);
+    const int st = has_pivots(h->twin) ? basker_refactor(h->twin, h->d_vals64, s)
+                                       : basker_factor(h->twin, h->d_vals64, s);
     h->use64 = true;
     h->info.ir_fallbacks++;
     if (st != BASKER_OK) h->info.failed_column = h->twin->info.failed_column;
@@ -1832,7 +1863,7 @@ int basker_factor(basker_t h, const double *values_dev, void *stream)
 {
     if (!h || (!values_dev && h->pl.nnz > 0)) return BASKER_ERR_INVALID_ARG;
     cudaSetDevice(h->device);
-    h->factored = false;
+    h->factored = h->pivots_kept = false;
     cudaStream_t s = (cudaStream_t)stream;
     if (h->opt.precision && h->pl.nnz > 0)
         CU(cudaMemcpyAsync(h->d_vals64, values_dev, sizeof(double) * (size_t)h->pl.nnz, cudaMemcpyDeviceToDevice, s));
@@ -1846,8 +1877,9 @@ int basker_factor(basker_t h, const double *values_dev, void *stream)
 int basker_refactor(basker_t h, const double *values_dev, void *stream)
 {
     if (!h || (!values_dev && h->pl.nnz > 0)) return BASKER_ERR_INVALID_ARG;
-    if (!h->factored) return BASKER_ERR_NOT_FACTORED;
+    if (!has_pivots(h)) return BASKER_ERR_NOT_FACTORED;
     cudaSetDevice(h->device);
+    h->pivots_kept = false;
     cudaStream_t s = (cudaStream_t)stream;
     if (h->opt.precision && h->pl.nnz > 0)
         CU(cudaMemcpyAsync(h->d_vals64, values_dev, sizeof(double) * (size_t)h->pl.nnz, cudaMemcpyDeviceToDevice, s));
@@ -1899,7 +1931,7 @@ int basker_refactor_solve_host(basker_t h, const double *values_host, int32_t nr
     }
     CU(cudaMemcpyAsync(h->d_vals, values_host, sizeof(double) * (size_t)h->pl.nnz, cudaMemcpyHostToDevice, s));
     if (nrhs > 0) CU(cudaMemcpyAsync(h->d_b, b_host, sizeof(double) * n * (size_t)nrhs, cudaMemcpyHostToDevice, s));
-    int st = h->factored ? basker_refactor(h, h->d_vals, stream) : basker_factor(h, h->d_vals, stream);
+    int st = has_pivots(h) ? basker_refactor(h, h->d_vals, stream) : basker_factor(h, h->d_vals, stream);
     if (st != BASKER_OK) return st;
     if (nrhs > 0) {
         TRY(basker_solve(h, nrhs, h->d_b, (int32_t)n, h->d_x, (int32_t)n, stream));
@@ -2019,7 +2051,7 @@ int basker_export(basker_t h, int32_t *prow, int64_t *Lp, int32_t *Li, double *L
 int basker_autotune(basker_t h, const double *values_dev, const double *b_dev, void *stream)
 {
     if (!h || (!values_dev && h->pl.nnz > 0) || (!b_dev && h->pl.n > 0)) return BASKER_ERR_INVALID_ARG;
-    if (!h->factored) return BASKER_ERR_NOT_FACTORED;
+    if (!has_pivots(h)) return BASKER_ERR_NOT_FACTORED;
     if (h->pl.n == 0) return BASKER_OK;
     cudaSetDevice(h->device);
     cudaStream_t s = (cudaStream_t)stream;

@@ -1,0 +1,62 @@
+"""The library's host code when a call of the runtime or a kernel's status reports a
+failure, without a GPU: the library runs over a fake CUDA runtime (fake_cudart.c) in a
+process of its own."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+from paper_1601_05725_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if cc is None or shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("no C or CUDA compiler")
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run([cc, "-O1", "-shared", "-fPIC", os.path.join(ROOT, "tests", "fake_cudart.c"), "-o", so], check=True)
+    return so
+
+
+def run(fake, body):
+    """``body`` in a process over the fake runtime."""
+    r = subprocess.run([sys.executable, "-c", "from tests.host_driver import *\n"
+                        "from paper_1601_05725_gb300 import inputs as I\n" + body],
+                       env=dict(os.environ, LD_PRELOAD=fake, PYTHONPATH=ROOT), cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+PROBLEMS = {
+    "grid": "I.grid_problem(3, k=40, depth=2)",
+    "netlist": "I.netlist_problem(4, n_small=30, m_netlist=3000, depth=2)",
+    "blocks": "I.block_diagonal_problem(5, nblocks=20, size_range=(1, 60))",
+}
+
+
+@pytest.mark.parametrize("name,switch,grown", [
+    (name, switch, grown) for name in sorted(PROBLEMS) for switch in (0, 1, 2, 3) for grown in (False, True)
+    if not (grown and name == "blocks" and switch % 2)])      # their stored-pattern pass needs no room
+def test_wait_that_gave_up_in_a_refactorization(fake, name, switch, grown):
+    """No solve with factors that are half new; a refactorization may follow, and starts
+    from no stored pattern.  The same when the factors had been given more room."""
+    run(fake, f"""
+h = Host({PROBLEMS[name]}, refactor_switch={switch})
+assert h.factor() == OK and h.solve() == OK and h.refactor() == OK and h.solve() == OK
+if {grown}:
+    fake.fake_status(0, CAPACITY, 1)
+    fake.fake_status(1, GAVE_UP, 1)
+else:
+    fake.fake_status(0, GAVE_UP, 1)
+assert h.refactor() == TIMEOUT
+assert h.solve() == NOT_FACTORED
+launched()
+assert h.refactor() == OK
+assert "bk_static_kernel" not in launched()
+assert h.solve() == OK and h.refactor() == OK and h.solve() == OK
+""")
