@@ -884,7 +884,10 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bo
             tend(h, s);
             h->launches++;
         }
-        if (h->lv_ncols[l] > 0) {
+        // staged: the leaves' part of all levels' columns goes ahead, whether or not a
+        // separator of level 1 has rows
+        const bool ahead = td_smem && h->td.loff && l == 1;
+        if (h->lv_ncols[l] > 0 || ahead) {
             // on the stored patterns; what fails that by the reach, nodes in parallel;
             // what outgrows its logs by the reach in one warp
             const bk_dev dl = level_dev(h, l);
@@ -895,7 +898,7 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bo
             // the reach with its nodes in parallel takes less)
             const bk_desc_par par = stored && l < h->df_par.size() && !td_smem ? h->df_par[l] : bk_desc_par{};
             CU(cudaMemsetAsync(cnt, 0, 16 * sizeof(int32_t), s));
-            tbeg(h, KT_DESC, s, (par.smem > 0) + (td_smem > 0) + 1);
+            tbeg(h, KT_DESC, s, (par.smem > 0) + (td_smem > 0) + (ncols > 0));
             if (par.smem) {
                 bk_launch_desc_fast(dl, list, ncols, cnt + 5, h->df_redo, cnt + 7, par, s);
                 CU(cudaGetLastError());
@@ -904,8 +907,8 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bo
                 h->launches++;
             }
             if (td_smem) {
-                // staged: the leaves' part of all levels' columns first, with level 1's whole
-                const int stage = !h->td.loff ? 0 : l == 1 ? 1 : 2;
+                // the stage that goes ahead takes level 1's columns whole
+                const int stage = !h->td.loff ? 0 : ahead ? 1 : 2;
                 bk_launch_tdesc(dl, h->td, stage == 1 ? h->td_cols : list, stage == 1 ? h->td_ncols : ncols, cnt + 11, nlist,
                                 h->td_over, cnt + 12, td_smem, stage, stage == 2 ? h->td_first[l] : 0, s);
                 CU(cudaGetLastError());
@@ -913,10 +916,12 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bo
                 nlist = cnt + 12;
                 h->launches++;
             }
-            bk_launch_gp_desc(dl, list, ncols, cnt + 3, s, nlist);
-            CU(cudaGetLastError());
+            if (ncols > 0) {
+                bk_launch_gp_desc(dl, list, ncols, cnt + 3, s, nlist);
+                CU(cudaGetLastError());
+                h->launches++;
+            }
             tend(h, s);
-            h->launches++;
         }
         for (int g = 0; g < BK_DENSE_GROUPS; g++) {
             if (h->lv_ndense[g][l] == 0) continue;

@@ -60,3 +60,14 @@ assert h.refactor() == OK
 assert "bk_static_kernel" not in launched()
 assert h.solve() == OK and h.refactor() == OK and h.solve() == OK
 """)
+
+
+def test_stages_above_an_empty_level(fake):
+    """The stage that goes ahead is launched although no separator of level 1 has rows."""
+    run(fake, """
+from tests.nd_cases import nd_problem
+h = Host(nd_problem(5, [300, 300, 0, 300, 300, 0, 3], chain=True))
+launched()
+assert h.factor() == OK
+assert launched().count("bk_tdesc_kernel") == 2
+""")
