@@ -39,7 +39,7 @@ struct basker_s {
     bool settled = false;        // the last refactorization moved no pivot
     bool patterns_hold = true;   // the stored patterns are a finished factorization's (or the symbolic ones):
                                  // a stored-pattern pass may start from them
-    bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once from then on
+    bool many_rejects = false;   // a stored-pattern pass rejected too many pivots: the teams at once, until they move few
     // separators whose in-node phase runs as one dense elimination, by kernel and cluster size
     // (bk_dense_node_group)
     std::vector<int32_t *> lv_dense[BK_DENSE_GROUPS];
@@ -1412,7 +1412,9 @@ int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool 
     if (st == BASKER_OK) {
         note_repair(h);
         h->settled = pref_mode && (first ? h->h_status->static_fail : h->h_status->repaired) == 0;
+        // (back when the teams alone have moved few pivots: the previous ones hold again)
         if (first && h->h_status->static_fail > many) h->many_rejects = true;
+        else if (!first && pref_mode && h->h_status->repaired <= many) h->many_rejects = false;
     }
     return st;
 }

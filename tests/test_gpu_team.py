@@ -112,3 +112,24 @@ def test_fp32_repair_equals_rounds():
         np.testing.assert_array_equal(a.indptr, b.indptr)
         np.testing.assert_array_equal(a.indices, b.indices)
         np.testing.assert_array_equal(a.data, b.data)
+
+
+def test_stored_patterns_serve_again_after_a_jump():
+    """After one refactorization that rejects many pivots, a sequence that repeats is
+    back on the stored patterns; the factors are the oracle's throughout."""
+    prob = I.grid_problem(5, k=61, depth=2)
+    o = oracle.OracleLU(prob)
+    assert o.factor(tau=0.3) == "OK"
+    f = o.factors()
+    h = basker.Handle.from_problem(prob, tau=0.3)
+    h.factor(_dev(prob.values))
+    stored = []
+    for k, sigma in ((1, 0.05), (1, 0.05), (1, 0.05), (2, 1.0), (2, 1.0), (2, 1.0)):
+        v = I.refactor_values(prob, k, sigma=sigma)
+        assert o.factor(v, tau=0.3, pref=f.prow) == "OK"
+        f = o.factors()
+        h.info()
+        h.refactor(_dev(v))
+        stored.append(h.info()["kernel_calls"]["static_refactor"])
+        _same(h, f)
+    assert stored == [1, 0, 1, 1, 0, 1]

@@ -71,3 +71,23 @@ launched()
 assert h.factor() == OK
 assert launched().count("bk_tdesc_kernel") == 2
 """)
+
+
+def test_stored_patterns_serve_again_after_a_jump(fake):
+    """A pass that rejects too many pivots turns the stored patterns off until the teams
+    alone have moved few."""
+    run(fake, """
+h = Host(I.grid_problem(3, k=61, depth=2))
+assert h.factor() == OK
+def stored():
+    launched()
+    assert h.refactor() == OK
+    return "bk_static_kernel" in launched()
+assert stored()
+fake.fake_status(0, REJECTED, 1000)
+assert stored()
+fake.fake_status(0, MOVED, 1000)
+assert not stored()          # the values jump again
+assert not stored()          # the pivots of before hold
+assert stored() and stored()
+""")
