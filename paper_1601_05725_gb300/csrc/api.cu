@@ -1419,6 +1419,31 @@ int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool 
     return st;
 }
 
+// The team kernel packs the place of an L column into 31 bits.
+bool teams_fit(basker_t h) { return h->team_path && h->d.lpool_end < INT32_MAX; }
+
+// The factors given more room and computed anew, until they fit: by teams, or by the
+// complete pass once the arena is too large for them.
+int grow_and_factor(basker_t h, cudaStream_t s, int pref_mode)
+{
+    int st = -1;
+    for (int tries = 0; st == -1 && tries < 16; tries++) {
+        TRY(regrow(h));
+        TRY(reset_status(h, s));
+        if (teams_fit(h)) {
+            bool stored = false;
+            st = factor_by_teams(h, s, pref_mode, false, stored);
+        } else {
+            h->schedule_valid = h->settled = false;
+            h->order_stale = true;
+            TRY(launch_full_gp(h, s, pref_mode));
+            st = read_status(h, s);
+            h->patterns_hold = st == BASKER_OK;
+        }
+    }
+    return st;
+}
+
 int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
 {
     h->launches = 0;
@@ -1433,7 +1458,7 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         CU(cudaMemcpyAsync((void *)h->d.pref, h->d.prow, sizeof(int32_t) * (size_t)h->pl.n,
                            cudaMemcpyDeviceToDevice, s));
         // options.refactor_switch 0, or 2 (the complete pass at once)
-        const bool teams = h->team_path && h->d.lpool_end < INT32_MAX && h->opt.refactor_switch % 2 == 0;
+        const bool teams = teams_fit(h) && h->opt.refactor_switch % 2 == 0;
         const bool from_patterns = !teams && h->patterns_hold;
         if (from_patterns) {
             if (!h->schedule_valid) TRY(compute_schedule(h, s));
@@ -1452,12 +1477,7 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
             const bool first = (h->stored_first || h->settled) && h->patterns_hold && !h->many_rejects &&
                                h->opt.refactor_switch == 0;
             st = factor_by_teams(h, s, 1, first, stored);
-            for (int tries = 0; st == -1 && tries < 16; tries++) {
-                TRY(regrow(h));
-                TRY(reset_status(h, s));
-                stored = false;
-                st = factor_by_teams(h, s, 1, false, stored);
-            }
+            if (st == -1) st = grow_and_factor(h, s, 1);
             if (st == BASKER_OK && h->opt.refactor_switch == 2 && h->h_status->repaired > 0) {
                 h->info.full_refactors++;
                 h->info.last_rounds = 0;
@@ -1501,7 +1521,7 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         return BASKER_OK;
     }
     int st = BK_SWITCH_TO_FULL;
-    if (h->team_path && h->d.lpool_end < INT32_MAX) {
+    if (teams_fit(h)) {
         // from the symbolic arena (natural pivots and patterns) when it is there:
         // the stored-pattern pass first, or at least the separators' patterns
         bool stored = h->sym_Li && h->sym_ver == h->arena_ver && !h->static_factor_off && h->lv_tasks.size() > 1;
@@ -1523,11 +1543,9 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
                 h->static_factor_off = true;
             }
         }
-        for (int tries = 0; st == -1 && tries < 16; tries++) {
-            TRY(regrow(h));
-            TRY(reset_status(h, s));
+        if (st == -1) {
+            st = grow_and_factor(h, s, 0);
             stored = false;
-            st = factor_by_teams(h, s, 0, false, stored);
         }
         if (st == BASKER_OK) {
             if (stored) h->info.static_factors++;

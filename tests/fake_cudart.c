@@ -7,6 +7,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/mman.h>
 
 typedef struct { unsigned x, y, z; } dim3_t;
 enum { OK = 0, OUT_OF_MEMORY = 2 };
@@ -16,6 +17,8 @@ static int64_t cap = INT64_MAX, held;       /* bytes of device memory: all there
 static int status_reads;                    /* status words read so far */
 static struct { int at, word, value; } plant[16];   /* those to change: a 32-bit word, and what to put there */
 static int nplants;
+static size_t ints_bytes;                   /* size of the copy to replace, and the value its ints get */
+static int ints_value, ints_times;
 static char launched[1 << 16];              /* names of the kernels launched since the last question */
 
 void fake_cap(int64_t bytes) { cap = bytes; }
@@ -30,6 +33,14 @@ void fake_status(int skip, int word, int value)
     nplants = (nplants + 1) % 16;
 }
 
+/* The next `times` synchronous copies of `bytes` bytes to the host read as ints of `value`. */
+void fake_ints(int64_t bytes, int value, int times)
+{
+    ints_bytes = (size_t)bytes;
+    ints_value = value;
+    ints_times = times;
+}
+
 const char *fake_launched(void)
 {
     static char out[sizeof launched];
@@ -40,6 +51,7 @@ const char *fake_launched(void)
 
 /* ---- memory */
 struct block { void *p; int64_t bytes; };
+enum { LARGE = 64 << 20 };                  /* from here on address space only, until it is written */
 static struct block *blocks;
 static size_t nblocks, room;
 
@@ -48,7 +60,12 @@ int cudaMalloc(void **p, size_t bytes)
     *p = NULL;
     if (held + (int64_t)bytes > cap) return OUT_OF_MEMORY;
     if (nblocks == room) blocks = realloc(blocks, (room = room ? 2 * room : 256) * sizeof *blocks);
-    *p = calloc(bytes ? bytes : 1, 1);
+    if (bytes >= LARGE) {
+        *p = mmap(NULL, bytes, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+        if (*p == MAP_FAILED) *p = NULL;
+    } else {
+        *p = calloc(bytes ? bytes : 1, 1);
+    }
     if (!*p) return OUT_OF_MEMORY;
     blocks[nblocks].p = *p;
     blocks[nblocks++].bytes = (int64_t)bytes;
@@ -60,9 +77,11 @@ int cudaFree(void *p)
 {
     for (size_t i = 0; p && i < nblocks; i++)
         if (blocks[i].p == p) {
+            const size_t bytes = (size_t)blocks[i].bytes;
             held -= blocks[i].bytes;
             blocks[i] = blocks[--nblocks];
-            free(p);
+            if (bytes >= LARGE) munmap(p, bytes);
+            else free(p);
             break;
         }
     return OK;
@@ -71,12 +90,20 @@ int cudaFree(void *p)
 int cudaMallocHost(void **p, size_t bytes) { *p = calloc(bytes ? bytes : 1, 1); return OK; }
 int cudaFreeHost(void *p) { free(p); return OK; }
 
-int cudaMemcpy(void *d, const void *s, size_t n, int kind) { (void)kind; if (n) memmove(d, s, n); return OK; }
+int cudaMemcpy(void *d, const void *s, size_t n, int kind)
+{
+    if (n) memmove(d, s, n);
+    if (kind == 2 && ints_times > 0 && n == ints_bytes) {
+        for (size_t i = 0; i < n / 4; i++) ((int32_t *)d)[i] = ints_value;
+        ints_times--;
+    }
+    return OK;
+}
 
 int cudaMemcpyAsync(void *d, const void *s, size_t n, int kind, void *stream)
 {
     (void)stream;
-    cudaMemcpy(d, s, n, kind);
+    if (n) memmove(d, s, n);
     if (kind == 2 && n == 40) {              /* device to host: the status word of a call */
         for (int i = 0; i < nplants; i++)
             if (plant[i].at == status_reads) ((int32_t *)d)[plant[i].word] = plant[i].value;

@@ -14,6 +14,7 @@ CAPACITY, GAVE_UP, REJECTED, MOVED = 2, 3, 4, 8
 fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
 fake.fake_held.restype = ctypes.c_int64
 fake.fake_cap.argtypes = [ctypes.c_int64]
+fake.fake_ints.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int]
 fake.fake_launched.restype = ctypes.c_char_p
 
 

@@ -91,3 +91,36 @@ assert not stored()          # the values jump again
 assert not stored()          # the pivots of before hold
 assert stored() and stored()
 """)
+
+
+@pytest.mark.parametrize("again", [False, True])
+def test_arena_that_outgrows_the_teams(fake, again):
+    """Room for the factors that grows past 2^31 entries of L: the complete pass, not the
+    teams, whose records hold 31 bits of a place."""
+    run(fake, f"""
+sizes = np.full(16, 15000)
+n = int(sizes.sum())
+first = np.isin(np.arange(n), np.cumsum(sizes) - sizes)
+r = np.concatenate([np.arange(n), np.flatnonzero(~first)])          # diagonal, and the row below
+c = np.concatenate([np.arange(n), np.flatnonzero(~first) - 1])
+at = np.lexsort((r, c))
+colptr = np.concatenate([[0], np.cumsum(np.bincount(c, minlength=n))])
+p = I.Problem("blocks", n, colptr, r[at], np.ones(r.size), np.arange(n), np.arange(n),
+              np.concatenate([[0], np.cumsum(sizes)]))
+h = Host(p)
+assert h.status == OK
+call = h.factor
+if {again}:
+    assert h.factor() == OK
+    call = h.refactor
+launched()
+# every column of L out of room, five times: 10, 104, 480, 1,984, 8,000 entries, then all a block can have
+for k in range(5):
+    fake.fake_status(k, CAPACITY, 1)
+fake.fake_ints(4 * n, 1, 5)
+assert call() == OK
+seen = launched()
+assert seen.count("bk_team_kernel") == 5 and seen.count("bk_gp_task_kernel") == 1, seen
+assert h.solve() == OK and h.refactor() == OK and h.solve() == OK
+assert "bk_team_kernel" not in launched()
+""")
