@@ -75,6 +75,7 @@ struct basker_s {
     int32_t *td_cols = nullptr;
     int32_t td_ncols = 0;
     int32_t *td_over = nullptr;
+    bool td_ready = false;           // all of the above is there
     // the arena as the symbolic pass left it (natural pivots, symbolic pattern and
     // schedule): a factorization first tries the stored-pattern path from it
     int32_t *sym_Li = nullptr, *sym_Ui = nullptr, *sym_n = nullptr;   // sym_n: 8 arrays of n ints
@@ -167,12 +168,21 @@ void tflush(basker_t h)
     h->pending.clear();
 }
 
+void release_tdesc(basker_t h);
+
 template <typename T>
 int dalloc(basker_t h, T **p, size_t count, bool zero = false)
 {
     *p = nullptr;
     size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-    if (cudaMalloc((void **)p, bytes) != cudaSuccess) {
+    cudaError_t e = cudaMalloc((void **)p, bytes);
+    if (e != cudaSuccess && h->td_ready) {
+        // the separator columns' logs are the handle's only memory it can do without
+        cudaGetLastError();
+        release_tdesc(h);
+        e = cudaMalloc((void **)p, bytes);
+    }
+    if (e != cudaSuccess) {
         cudaGetLastError();
         return BASKER_ERR_OOM;
     }
@@ -200,6 +210,22 @@ void dfree(basker_t h, void *p)
     }
     std::lock_guard<std::mutex> lk(g_capture_mu);
     cudaFree(p);
+}
+
+// The columns' logs and vectors given back: the reach in one warp a column takes every
+// level from now on.
+void release_tdesc(basker_t h)
+{
+    h->td_ready = false;
+    bk_tdesc_dev &t = h->td;
+    dfree(h, t.slot); dfree(h, t.l); dfree(h, t.m); dfree(h, t.x); dfree(h, t.state);
+    dfree(h, (void *)t.loff); dfree(h, (void *)t.xoff); dfree(h, h->td_cols); dfree(h, h->td_over);
+    unsigned long long *const link = t.link;
+    t = bk_tdesc_dev{};
+    t.link = link;
+    h->td_cols = h->td_over = nullptr;
+    h->td_ncols = 0;
+    std::fill(h->td_smem.begin(), h->td_smem.end(), (size_t)0);
 }
 
 cudaError_t device_sync()
@@ -429,7 +455,8 @@ int setup_teams(basker_t h)
 }
 
 // The reach of separator columns with their descendant nodes in parallel, where the
-// column's bitmaps fit on chip.
+// column's bitmaps fit on chip and the device has the room: a handle does without (one
+// warp a column) when its own or a later allocation finds none.
 int setup_tdesc(basker_t h)
 {
     const bk_plan &pl = h->pl;
@@ -500,19 +527,29 @@ int setup_tdesc(basker_t h)
         const int64_t words = (int64_t)(worst / 4) + 8;
         if (!all.empty() && worst <= BK_TDESC_SMEM &&
             loff.back() * 20 + xoff.back() * 8 + words * 4 * (int64_t)all.size() <= ((int64_t)1 << 30)) {
-            h->td_ncols = (int32_t)all.size();
-            h->td.words = (int32_t)words;
-            for (size_t l = 1; l < nl; l++) h->td_smem[l] = worst;
-            TRY(upload(h, &h->td_cols, all));
-            TRY(upload(h, (int64_t **)&h->td.loff, loff));
-            TRY(upload(h, (int64_t **)&h->td.xoff, xoff));
-            TRY(dalloc(h, &h->td.x, (size_t)xoff.back(), true));
-            TRY(dalloc(h, &h->td.state, (size_t)words * all.size(), true));
-            TRY(dalloc(h, &h->td.slot, (size_t)loff.back()));
-            TRY(dalloc(h, &h->td.l, (size_t)loff.back()));
-            TRY(dalloc(h, &h->td.m, (size_t)loff.back()));
-            TRY(dalloc(h, &h->td_over, (size_t)pl.n));
-            return BASKER_OK;
+            const int32_t nodes = h->td.nodes;
+            auto staged = [&]() {
+                TRY(upload(h, &h->td_cols, all));
+                TRY(upload(h, (int64_t **)&h->td.loff, loff));
+                TRY(upload(h, (int64_t **)&h->td.xoff, xoff));
+                TRY(dalloc(h, &h->td.x, (size_t)xoff.back(), true));
+                TRY(dalloc(h, &h->td.state, (size_t)words * all.size(), true));
+                TRY(dalloc(h, &h->td.slot, (size_t)loff.back()));
+                TRY(dalloc(h, &h->td.l, (size_t)loff.back()));
+                TRY(dalloc(h, &h->td.m, (size_t)loff.back()));
+                return dalloc(h, &h->td_over, (size_t)pl.n);
+            };
+            const int st = staged();
+            if (st == BASKER_OK) {
+                h->td_ncols = (int32_t)all.size();
+                h->td.words = (int32_t)words;
+                for (size_t l = 1; l < nl; l++) h->td_smem[l] = worst;
+                h->td_ready = true;
+                return BASKER_OK;
+            }
+            release_tdesc(h);
+            if (st != BASKER_ERR_OOM) return st;
+            h->td.nodes = nodes;             // no room for the stages
         }
     }
     if (most == 0) return BASKER_OK;
@@ -520,11 +557,19 @@ int setup_tdesc(basker_t h)
     h->td.cap = (int32_t)(std::min<int64_t>(std::max<int64_t>(4 * rows, 16384), 262144) + 63) & ~63;
     h->td.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>({most, 304, ((int64_t)128 << 20) / ((int64_t)h->td.cap * 20)}));
     sizes();
+    auto whole = [&]() {
+        TRY(dalloc(h, &h->td.slot, (size_t)h->td.cap * (size_t)h->td.blocks));
+        TRY(dalloc(h, &h->td.l, (size_t)h->td.cap * (size_t)h->td.blocks));
+        TRY(dalloc(h, &h->td.m, (size_t)h->td.cap * (size_t)h->td.blocks));
+        return dalloc(h, &h->td_over, (size_t)pl.n);
+    };
+    const int st = whole();
+    if (st != BASKER_OK) {
+        release_tdesc(h);
+        return st == BASKER_ERR_OOM ? BASKER_OK : st;
+    }
     for (size_t l = 1; l < nl; l++) h->td_smem[l] = on[l] && sm[l] <= BK_TDESC_SMEM ? sm[l] : 0;
-    TRY(dalloc(h, &h->td.slot, (size_t)h->td.cap * (size_t)h->td.blocks));
-    TRY(dalloc(h, &h->td.l, (size_t)h->td.cap * (size_t)h->td.blocks));
-    TRY(dalloc(h, &h->td.m, (size_t)h->td.cap * (size_t)h->td.blocks));
-    TRY(dalloc(h, &h->td_over, (size_t)pl.n));
+    h->td_ready = true;
     return BASKER_OK;
 }
 

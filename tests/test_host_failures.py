@@ -124,3 +124,58 @@ assert seen.count("bk_team_kernel") == 5 and seen.count("bk_gp_task_kernel") == 
 assert h.solve() == OK and h.refactor() == OK and h.solve() == OK
 assert "bk_team_kernel" not in launched()
 """)
+
+
+@pytest.mark.parametrize("make", [
+    "I.netlist_problem(94, n_small=60, m_netlist=20000, depth=2)",                      # in stages
+    "I.netlist_problem(91, n_small=40, m_netlist=6000, depth=1, n_rails=5, rail_deg=(2200, 4000))",   # columns whole
+])
+def test_no_room_for_the_separator_columns_logs(fake, make):
+    """The logs are room a handle can do without: it is made, grows and factors as long as
+    the rest fits."""
+    run(fake, f"""
+import ctypes
+p = {make}
+def size(h):
+    i = basker.Info()
+    assert h.L.basker_info(h.h, ctypes.byref(i)) == OK and i.device_bytes == fake.fake_held()
+    return i.device_bytes
+h = Host(p)
+full = size(h)
+launched()
+assert h.factor() == OK and "bk_tdesc_kernel" in launched()
+h.free()
+assert fake.fake_held() == 0
+def made(cap):
+    fake.fake_cap(cap)
+    h = Host(p)
+    if h.status == OK:
+        assert size(h) <= cap and h.factor() == OK
+        h.has_logs = "bk_tdesc_kernel" in launched()
+    return h
+# the least room that a handle is made in (it has no logs), by bisection
+lo, hi = 0, full
+while hi - lo > 4096:
+    mid = (lo + hi) // 2
+    h = made(mid)
+    lo, hi = (lo, mid) if h.status == OK else (mid, hi)
+    h.free()
+assert hi < full - 4096, "the handle's own size is the least it is made in"
+h = made(hi)
+assert not h.has_logs
+h.free()
+for step in range(1, 8):                 # the logs' own allocations fail, or a later one does
+    h = made(hi + (full - hi) * step // 8)
+    assert h.status == OK
+    h.free()
+h = made(full)
+assert h.has_logs
+# a later call wants room: the logs go
+fake.fake_cap(full + 8 * p.n)
+assert h.solve() == OK and size(h) < full
+launched()
+assert h.refactor() == OK and "bk_tdesc_kernel" not in launched()
+h.free()
+fake.fake_cap(1 << 20)
+assert Host(p).status == OOM and fake.fake_held() == 0
+""")
