@@ -213,6 +213,8 @@ __global__ void __launch_bounds__(DR_THREADS, 1) bk_dense_rows_kernel(bk_dev d, 
         if (sl < lsp && ((bits[(int64_t)k * nrw + (sl >> 5)] >> (sl & 31)) & 1u)) v = A[(int64_t)k * lsp + sl];
         loc[(int64_t)rl * ld + k] = v;
     }
+    // an earlier failure: the first messages say so, and no step runs
+    if (rank == 0 && tx == 0 && should_stop(d, tid, T.lo)) S.stopreq = 1;
     cl.sync();
 
     // L(:, step j) from lcol, its pivot slot pp (the last DR_DIV warps)
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) bk_dense_rows_kernel(bk_dev d, 
                     S.cnt = carry;
                     S.lover = lbs[k] + carry - 1 > les[k];
                 }
-            } else if (wid == DR_WARPS - 1 && rank == 0 && lane == 0 && (k & 15) == 0) {
+            } else if (wid == DR_WARPS - 1 && rank == 0 && lane == 0 && (k & 15) == 0 && k > 0) {
                 if (should_stop(d, tid, c)) S.stopreq = 1;
             }
             if (k > 0) {
