@@ -972,7 +972,7 @@ int launch_separators(basker_t h, cudaStream_t s, int pref_mode, bool stored, bo
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], h->opt.tau, pref_mode,
-                                  g, s);
+                                  g, h->opt.wait_budget_cycles, s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;
@@ -1008,7 +1008,7 @@ int launch_full_gp(basker_t h, cudaStream_t s, int pref_mode)
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], tau, pref_mode,
-                                  g, s);
+                                  g, std::max<long long>(h->opt.wait_budget_cycles, BK_DENSE_WAIT), s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;
@@ -1113,7 +1113,8 @@ int launch_redo(basker_t h, cudaStream_t s)
                     if (dense[g].empty()) continue;
                     tbeg(h, KT_DENSE, s, 1);
                     bk_launch_dense_nodes(h->d, h->rd_tasks + at[g], (int32_t)dense[g].size(),
-                                          (dsm[g] + 15) & ~(size_t)15, tau, 1, g, s);
+                                          (dsm[g] + 15) & ~(size_t)15, tau, 1, g,
+                                          h->opt.wait_budget_cycles, s);
                     CU(cudaGetLastError());
                     tend(h, s);
                     h->launches++;
@@ -1226,7 +1227,7 @@ int launch_repair_path(basker_t h, cudaStream_t s)
             if (h->lv_ndense[g][l] == 0) continue;
             tbeg(h, KT_DENSE, s, 1);
             bk_launch_dense_nodes(h->d, h->lv_dense[g][l], h->lv_ndense[g][l], h->lv_dsmem[g][l], h->opt.tau, 1,
-                                  g, s);
+                                  g, h->opt.wait_budget_cycles, s);
             CU(cudaGetLastError());
             tend(h, s);
             h->launches++;

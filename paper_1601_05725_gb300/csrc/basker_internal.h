@@ -184,11 +184,15 @@ bool bk_dense_node_eligible(const bk_task &t);
 #define BK_DENSE_CLUSTER_MIN 64
 #define BK_DENSE_GROUPS 3
 int bk_dense_node_group(const bk_task &t);
+// budget: cycles of a wait for another block's message, after which the call times out.
+// The complete pass, which a factorization falls back on when a wait gave up, gives
+// them BK_DENSE_WAIT at least (about two seconds)
+#define BK_DENSE_WAIT (1ll << 32)
 void bk_launch_dense_nodes(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                           int pref_mode, int group, void *stream);
+                           int pref_mode, int group, long long budget, void *stream);
 size_t bk_dense_rows_smem(const bk_task &t, int cluster);
 void bk_launch_dense_rows(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                          int pref_mode, int cluster, void *stream);
+                          int pref_mode, int cluster, long long budget, void *stream);
 bool bk_task_fits_smem(const bk_task &t);
 
 // kernels (launchers), kernels_*.cu

@@ -464,11 +464,11 @@ bool bk_dense_node_eligible(const bk_task &T)
 }
 
 void bk_launch_dense_nodes(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                           int pref_mode, int group, void *stream)
+                           int pref_mode, int group, long long budget, void *stream)
 {
     if (ntasks <= 0) return;
     if (group < 2) {
-        bk_launch_dense_rows(d, task_ids, ntasks, smem, tau, pref_mode, group ? BK_DENSE_CLUSTER : 1, stream);
+        bk_launch_dense_rows(d, task_ids, ntasks, smem, tau, pref_mode, group ? BK_DENSE_CLUSTER : 1, budget, stream);
         return;
     }
     const int cluster = BK_DENSE_CLUSTER;

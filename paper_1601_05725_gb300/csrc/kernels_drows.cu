@@ -53,7 +53,6 @@ namespace {
 constexpr int DR_THREADS = 512;
 constexpr int DR_WARPS = DR_THREADS / 32;
 constexpr int DR_DIV = 4;                      // warps that divide
-constexpr long long DR_LIMIT = 1ll << 32;      // cycles of a wait, at most (about two seconds)
 
 struct DrShared {
     bk_task T;
@@ -61,7 +60,7 @@ struct DrShared {
     int flag[2];                         // a U region is full (by step parity)
     int nrows[2];                        // own rows of the step's L column (by step parity)
     int cnt, lover;                      // column k: entries of its pattern, L region too small
-    int stopreq;                         // block 0: an earlier failure elsewhere
+    int stopreq;                         // an earlier failure elsewhere (block 0), or this block's wait budget is spent
     int stop;                            // leave
     int ok, ps, hnext;                   // the step's pivot: found, its slot, in the next column's pattern
     unsigned long long xp;               // its value
@@ -112,11 +111,34 @@ __device__ __forceinline__ void dr_expect(const void *bar, int bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(dr_addr(bar)), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ bool dr_wait(const bk_dev &d, const void *bar, int parity)
+// A step's messages.  A wait longer than the budget times the call out, but the messages
+// are still taken: the block says so in its next one (stopreq), and every block leaves
+// after the same step, with nothing under way to one that has left.  Only a message that
+// never comes ends the wait itself, BK_DENSE_WAIT cycles later.  (The first look does not
+// block, so that a budget of a few cycles is noticed.)
+__device__ __forceinline__ bool dr_wait(const bk_dev &d, DrShared &S, const void *bar, int parity, long long budget)
 {
-    long long t0 = 0;
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(dr_addr(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    const long long t0 = clock64();
+    bool told = false;
     for (;;) {
-        uint32_t done;
+        const long long t = clock64() - t0;
+        if (t > budget) {
+            if (!told) {
+                atomicExch(&d.status->timeout, 1);
+                S.stopreq = 1;
+                told = true;
+            }
+            if (t - budget > BK_DENSE_WAIT) return false;
+        }
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
@@ -125,11 +147,6 @@ __device__ __forceinline__ bool dr_wait(const bk_dev &d, const void *bar, int pa
             : "r"(dr_addr(bar)), "r"(parity)
             : "memory");
         if (done) return true;
-        if (t0 == 0) t0 = clock64();
-        if (clock64() - t0 > DR_LIMIT) {
-            atomicExch(&d.status->timeout, 1);
-            return false;
-        }
     }
 }
 
@@ -147,7 +164,7 @@ __host__ __device__ inline size_t dr_bytes(int own, int lsp, int cn)
 
 template <typename V, int CN>
 __global__ void __launch_bounds__(DR_THREADS, 1) bk_dense_rows_kernel(bk_dev d, const int32_t *__restrict__ task_ids,
-                                                                   double tau, int pref_mode)
+                                                                   double tau, int pref_mode, long long budget)
 {
     V *const Lx = vals<V>(d.Lx);
     V *const Ux = vals<V>(d.Ux);
@@ -254,15 +271,16 @@ __global__ void __launch_bounds__(DR_THREADS, 1) bk_dense_rows_kernel(bk_dev d, 
             unsigned long long wmax = dr_max(best == INT_MAX ? 0 : kmax);
             best = __reduce_min_sync(BK_FULL, best != INT_MAX && kmax == wmax ? best : INT_MAX);
             bad = __any_sync(BK_FULL, bad);
+            const bool leave = *reinterpret_cast<const volatile int *>(&S.stopreq) != 0;
             if (lane < CN) {
                 dr_send(msg + b * (CN + 1) + rank, &S.mb1[b], lane,
                         best == INT_MAX ? 0ull : dr_word(loc[(best / CN) * ld + k]),
-                        (unsigned)best | (bad ? 1ull << 32 : 0ull) | (S.stopreq ? 1ull << 33 : 0ull));
+                        (unsigned)best | (bad ? 1ull << 32 : 0ull) | (leave ? 1ull << 33 : 0ull));
                 if (prefok && pr % CN == rank)
                     dr_send(msg + b * (CN + 1) + CN, &S.mb1[b], lane, dr_word(loc[(pr / CN) * ld + k]), 0ull);
             }
             // every block's best row: the pivot
-            bool ok = dr_wait(d, &S.mb1[b], par);
+            bool ok = dr_wait(d, S, &S.mb1[b], par, budget);
             if (__all_sync(BK_FULL, ok)) {
                 unsigned long long v = 0, meta = (unsigned)INT_MAX;
                 if (lane < CN) {
@@ -432,7 +450,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) bk_dense_rows_kernel(bk_dev d, 
                     if (in) rows[at + __popc(all & ((1u << lane) - 1u))] = rl;
                 }
                 // the step on the next column, as soon as the pivot row is there
-                go = dr_wait(d, &S.mb2[b], par);
+                go = dr_wait(d, S, &S.mb2[b], par, budget);
                 if (go && S.hnext) {
                     const unsigned long long mw = mrow[b * nown2 + k + 1];
                     const V m = dr_value<V>(mw);
@@ -539,7 +557,7 @@ size_t bk_dense_rows_smem(const bk_task &T, int cluster) { return dr_bytes(T.hi 
 
 // task_ids: nodes whose rows fit the shared memory of `cluster` blocks
 void bk_launch_dense_rows(const bk_dev &d, const int32_t *task_ids, int32_t ntasks, size_t smem, double tau,
-                          int pref_mode, int cluster, void *stream)
+                          int pref_mode, int cluster, long long budget, void *stream)
 {
     if (ntasks <= 0) return;
     static std::once_flag once;
@@ -563,7 +581,7 @@ void bk_launch_dense_rows(const bk_dev &d, const int32_t *task_ids, int32_t ntas
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto go = [&](auto kernel) { cudaLaunchKernelEx(&cfg, kernel, d, task_ids, tau, pref_mode); };
+    auto go = [&](auto kernel) { cudaLaunchKernelEx(&cfg, kernel, d, task_ids, tau, pref_mode, budget); };
     if (cluster == 1) {
         if (d.prec) go(bk_dense_rows_kernel<float, 1>);
         else go(bk_dense_rows_kernel<double, 1>);

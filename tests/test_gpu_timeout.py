@@ -6,6 +6,7 @@ import pytest
 import oracle
 from paper_1601_05725_gb300 import basker, build
 from paper_1601_05725_gb300 import inputs as I
+from tests.nd_cases import nd_problem
 
 pytestmark = pytest.mark.gpu
 
@@ -79,3 +80,26 @@ def test_after_a_wait_that_gave_up(make, switch):
     assert o.factor() == "OK"
     h.factor(_dev(prob.values))
     _same(h, o.factors())
+
+
+@pytest.mark.parametrize("m", [40, 100])         # one block, a cluster of blocks
+@pytest.mark.parametrize("switch", [0, 1, 3])
+def test_budget_of_the_separators_elimination(m, switch):
+    """Leaves of one row wait for nothing: only the elimination's messages do.  The budget
+    is theirs too, and a factorization falls back on a pass that gives them their time."""
+    prob = nd_problem(3, [1, 1, m])
+    o = oracle.OracleLU(prob)
+    assert o.factor() == "OK"
+    f = o.factors()
+    h = basker.Handle.from_problem(prob, wait_budget_cycles=1, refactor_switch=switch)
+    for _ in range(2):
+        h.factor(_dev(prob.values))
+        _same(h, f)
+        with pytest.raises(basker.BaskerError) as e:
+            h.refactor(_dev(prob.values))
+        assert e.value.name == "TIMEOUT"
+        _refused(lambda: h.solve(_dev(np.ones(prob.n))))
+    h = basker.Handle.from_problem(prob, refactor_switch=switch)
+    h.factor(_dev(prob.values))
+    h.refactor(_dev(prob.values))
+    _same(h, f)
