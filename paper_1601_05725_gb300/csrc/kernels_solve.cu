@@ -668,7 +668,9 @@ __device__ void sep_sweep_block(const bk_dev &d, const bk_solve_dev &s, int it, 
     for (int r = tid; r < m * rr && ok; r += SW_NT) {
         const U v = await_value<V>(d, part + r, budget);
         ok = v != SW::none;
-        if (zs == zsm) zs[r] = SW::value(v);
+        // in place too: the other threads read what this one stores before the barrier, not
+        // what another block has stored (a relaxed poll orders nothing)
+        zs[r] = SW::value(v);
     }
     if (__syncthreads_or(!ok)) return;
     BK_TPHASE0(tp);

@@ -7,6 +7,7 @@ import pytest
 import oracle
 from paper_1601_05725_gb300 import basker, build
 from paper_1601_05725_gb300 import inputs as I
+from tests.nd_cases import nd_problem
 
 pytestmark = pytest.mark.gpu
 
@@ -62,3 +63,20 @@ def test_solve_carries_non_finite_right_hand_sides(name):
     b.view(np.uint64)[prob.n - 7] = np.uint64(0xFFFFFFFFFFFFFFFF)
     x, xo = h.solve(torch.as_tensor(b, device="cuda")).cpu().numpy(), o.solve(b)
     np.testing.assert_array_equal(x, xo)          # NaN equal to NaN
+
+
+@pytest.mark.parametrize("m,nrhs", [(1025, 1), (1100, 3), (481, 32), (500, 33)])
+def test_separators_swept_in_place(m, nrhs):
+    """A separator with more values than a sweeper's shared memory holds (1,024 rows; 480
+    with 32 right-hand sides) is swept in global memory."""
+    import torch
+    prob = nd_problem(m, [7, 5, m], density=0.02)
+    o = oracle.OracleLU(prob)
+    assert o.factor() == "OK"
+    h = basker.Handle.from_problem(prob)
+    h.factor(torch.as_tensor(prob.values, device="cuda"))
+    rng = np.random.default_rng(nrhs)
+    for _ in range(3):
+        B = rng.standard_normal((prob.n, nrhs))
+        X = h.solve(torch.as_tensor(B, device="cuda")).cpu().numpy()
+        np.testing.assert_array_equal(X, o.solve(B).reshape(prob.n, nrhs))
