@@ -317,6 +317,7 @@ int upload_symbolic_pattern(basker_t h)
         // and computes the schedule of its pattern
         if (!h->d.iorder) TRY(upload(h, (int32_t **)&h->d.iorder, pl.iorder));
         h->order_is_symbolic = false;
+        h->order_stale = true;       // there is no order yet that the levels could keep
         return BASKER_OK;
     }
     std::vector<int32_t> Li((size_t)pl.lcap, 0), Ui((size_t)pl.ucap, 0);

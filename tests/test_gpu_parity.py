@@ -422,3 +422,29 @@ def test_wait_budget_gives_timeout_not_hang():
     h2.factor(_dev(prob.values))
     h2.refactor(_dev(prob.values))
     assert_same_factors(h2, o.factors())
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("factor_mode", [0, 1])
+def test_refactor_of_a_lower_triangle_sized_by_counts(mode, factor_mode):
+    """No column waits for another (U is its diagonal) and no schedule came with the
+    analysis: the stored-pattern pass still takes every column."""
+    rng = np.random.default_rng(5)
+    n = 300
+    M = np.tril(rng.uniform(0.1, 1.0, (n, n)) * (rng.random((n, n)) < 0.05), -1) + np.diag(rng.uniform(1.0, 2.0, n))
+    prob = H.make_problem(M, scramble_seed=5)
+    o = oracle.OracleLU(prob)
+    h = basker.Handle.from_problem(prob, symbolic_mode=mode, factor_mode=factor_mode)
+    assert o.factor() == "OK"
+    h.factor(_dev(prob.values))
+    assert_same_factors(h, o.factors())
+    for k in (1, 2):
+        v = I.refactor_values(prob, k, sigma=0.3)
+        assert o.factor(v, pref=o.factors().prow) == "OK"
+        h.refactor(_dev(v))
+        assert_same_factors(h, o.factors())
+    v[0] = np.nan
+    assert o.factor(v, pref=o.factors().prow) == "NAN"
+    with pytest.raises(basker.BaskerError) as e:
+        h.refactor(_dev(v))
+    assert e.value.name == "NAN"

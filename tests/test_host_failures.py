@@ -179,3 +179,18 @@ h.free()
 fake.fake_cap(1 << 20)
 assert Host(p).status == OOM and fake.fake_held() == 0
 """)
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_first_schedule_of_a_handle_without_patterns(fake, mode):
+    """A handle from counts alone has no claim order before its first factorization, so
+    that one is computed, not checked."""
+    run(fake, f"""
+n = 8
+p = I.Problem("diagonal", n, np.arange(n + 1), np.arange(n), np.ones(n), np.arange(n), np.arange(n), np.array([0, n]))
+h = Host(p, symbolic_mode={mode}, factor_mode=1)
+launched()
+assert h.factor() == OK
+seen = launched()
+assert "bk_levels_kernel" in seen and "bk_level_check_kernel" not in seen
+""")
