@@ -1429,6 +1429,9 @@ int refactor_by_rounds(basker_t h, cudaStream_t s)
 int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool &stored)
 {
     const int32_t many = std::max(16, h->pl.n / 200);
+    // A failure in a leaf or block does not end the call: a separator's column may come
+    // before it and fail as well (a BTF block behind the ND block), and the first is named.
+    auto unfinished = [](int st) { return st != BASKER_OK && st != BASKER_ERR_SINGULAR && st != BASKER_ERR_NAN; };
     if (first) {
         if (!h->schedule_valid) TRY(compute_schedule(h, s));
         TRY(static_pass(h, s));
@@ -1437,13 +1440,13 @@ int factor_by_teams(basker_t h, cudaStream_t s, int pref_mode, bool first, bool 
     TRY(launch_leaves(h, s, pref_mode, first));
     if (h->lv_tasks.size() > 1 && stored && !pref_mode && !first) {
         const int st = read_status(h, s);
-        if (st != BASKER_OK) return st;
+        if (unfinished(st)) return st;
         stored = h->h_status->repaired <= many;
     }
     bool same = false;
     if (first && !h->stored_first && h->lv_tasks.size() > 1) {
         const int st = read_status(h, s);
-        if (st != BASKER_OK) {
+        if (unfinished(st)) {
             h->settled = h->patterns_hold = h->leaf_levels = false;
             h->order_stale = true;
             return st;
