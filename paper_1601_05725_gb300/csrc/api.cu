@@ -1552,6 +1552,9 @@ int factor_impl(basker_t h, const double *values, cudaStream_t s, bool refactor)
         } else {
             st = refactor_by_rounds(h, s);
         }
+        // rounds end at the first level that fails, and other levels may hold an earlier
+        // column that fails too: the complete pass names the first
+        if (from_patterns && (st == BASKER_ERR_SINGULAR || st == BASKER_ERR_NAN)) st = refactor_completely(h, s);
         if (st != BASKER_OK) {
             h->factored = false;
             if (st == BASKER_ERR_TIMEOUT) {

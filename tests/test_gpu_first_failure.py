@@ -92,3 +92,28 @@ def test_refactorization(tree, settled):
         assert o.factor() == "OK"
         h.factor(_dev(prob.values))
         _same(h, o.factors())
+
+
+@pytest.mark.parametrize("tree", sorted(TREES))
+@pytest.mark.parametrize("kw", [dict(refactor_switch=1), dict(refactor_switch=3), dict(factor_mode=1),
+                                dict(factor_mode=1, refactor_switch=3)], ids=str)
+def test_refactorization_without_teams(tree, kw):
+    """Rounds, the one-block repair and the column-by-column in-node phase; failures among
+    rejected pivots."""
+    prob, seps, blocks = _make(tree)
+    o = oracle.OracleLU(prob)
+    ptr = prob.nd_node_ptr
+    leaf = [int(ptr[0]) + 3, int(ptr[4]) + 2]
+    for bad in ([seps[0]] + blocks, [~seps[1]] + blocks, [seps[1]] + leaf, leaf[::-1] + blocks):
+        h = basker.Handle.from_problem(prob, **kw)
+        assert o.factor() == "OK"
+        h.factor(_dev(prob.values))
+        v = _failing(prob, I.refactor_values(prob, 1, sigma=0.7), bad)
+        status = o.factor(v, pref=o.factors().prow)
+        assert status != "OK"
+        with pytest.raises(basker.BaskerError) as e:
+            h.refactor(_dev(v))
+        assert (e.value.name, e.value.column) == (status, o.info_col)
+        assert o.factor() == "OK"
+        h.factor(_dev(prob.values))
+        _same(h, o.factors())
