@@ -359,12 +359,15 @@ def _measure(h, dvals, drhs, K, W, dev, flush, dist, world):
     return step_ms, xs.cpu().numpy(), info0, info1, (t0, t1)
 
 
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one
-# ncu capture of the kernel as it stands, by kernel kind and value width.  A kind
-# without a capture of its current code reports null.
-TRAFFIC = {}
-# sm__pipe_fp64_cycles_active (pct of peak) from the same captures
-FP64_PIPE = {}
+# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu
+# captures of the kernels as they stand, by kernel kind and value width (dense_node:
+# the mean of the four ND heights' launches).
+# A kind without a capture of its current code reports null.
+TRAFFIC = {("powergrid_316x316", "refactor_rounds", 8): 16.6e6, ("powergrid_316x316", "static_refactor", 8): 206.7e6,
+           ("powergrid_316x316", "dense_node", 8): 1.8e6, ("powergrid_316x316", "solve", 8): 102.7e6}
+# sm__pipe_fp64_cycles_active (pct of peak, of the SMs at work) from the same captures
+FP64_PIPE = {("powergrid_316x316", "refactor_rounds", 8): 17.5, ("powergrid_316x316", "static_refactor", 8): 32.0,
+             ("powergrid_316x316", "dense_node", 8): 42.7, ("powergrid_316x316", "solve", 8): 22.2}
 
 
 def _roofline(prob, info1, K, nnz_lu, vbytes, hbm):

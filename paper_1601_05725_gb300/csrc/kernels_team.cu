@@ -24,9 +24,9 @@
 // What bounds it: about 72 % of the columns of a netlist or grid leaf depend on
 // the column just before them (postordered subtrees), so the time is the task's
 // columns times the link from one decision to the next: the flag, the step's
-// entries (shared memory), the pivot search, a division; about 5,000 cycles, of
-// which an issue every 7.7 cycles a warp (dependent instructions) is the cause, not
-// memory (L2 0.05 %, DRAM 0.01 % of peak).  Measured against one warp walking the
+// entries (shared memory), the pivot search, a division; about 4,000 cycles by the
+// trace, 4,600 to 5,000 a column, of which an issue every 8 cycles a warp (dependent
+// instructions) is the cause, not memory (DRAM 0.02 % of peak).  Measured against one warp walking the
 // columns alone, a launch: leaves of 2,499 columns (20,011-row netlist) 5.5 ms, was
 // 44; of 4,685 columns (150,001 rows) 11.2 ms, was 87; 4,096 blocks of up to 1,024
 // rows 7.3 ms, was 41.
