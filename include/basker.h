@@ -54,7 +54,9 @@ typedef enum {
 typedef struct {
     double tau;                   /* pivot threshold in (0,1]; default 1e-3 */
     double slack;                 /* extra L/U capacity over the symbolic count; default 1.0 */
-    long long wait_budget_cycles; /* clock64 cycles any in-kernel wait may spin; default 2e10 */
+    long long wait_budget_cycles; /* clock64 cycles any in-kernel wait may spin; default 2e10.  (In
+                                     the complete pass, a factorization's last resort, the messages
+                                     of the separators' elimination have 2^32 at least.) */
     int factor_mode;              /* 0 (default): the in-node phase of an ND separator whose
                                      column state fits in shared memory runs as one dense
                                      right-looking elimination by a block of threads; 1: every
